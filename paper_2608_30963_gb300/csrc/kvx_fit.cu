@@ -14,17 +14,17 @@
 // Otherwise (fp32 caches, wider inputs):
 //   fit_rows_kernel builds X and Y for one pass of up to chunk tokens, then fit_gram_simt_kernel
 //   adds their products into the sums on the CUDA cores.
-// Solve (kvx_fit_solve): one CTA per group factors X^T X + lambda I = L L^T and runs the two
-//   triangular solves per output column: fit_solve_small_kernel in fp32 shared memory for
-//   in <= 256, handing the systems whose factor shows a condition number above 10^3 to
-//   fit_solve_kernel, which solves in double in global memory (and solves every system above
-//   in = 256).
+// Solve (kvx_fit_solve), in <= 256: a blocked Cholesky factor X^T X + lambda I = L L^T and the two
+//   triangular solves (kvx_fit_solve.cuh) in fp32, and again in pairs of floats (about 48 bits) for
+//   the systems whose factor shows a condition number above 10^3.  Wider systems: fit_solve_kernel,
+//   one CTA per group, in double in global memory.
 #include <math.h>
 #include <stdarg.h>
 #include <stdio.h>
 #include <string.h>
 
 #include "kvx_common.cuh"
+#include "kvx_fit_solve.cuh"
 #include "kvx_kernels.h"
 #include "kvx_tc_common.cuh"
 
@@ -35,10 +35,11 @@ constexpr int kFitTile = 32;
 constexpr int kFitThreads = 256;
 constexpr int kSolveThreads = 256;
 constexpr unsigned kFitNotPosDef = 0x20u;   // status bit: a system was not positive definite
-constexpr unsigned kFitSolvedDouble = 0x40u;   // status bit: ill-conditioned systems were solved in double
+constexpr unsigned kFitSolvedDouble = 0x40u;   // status bit: ill-conditioned systems were solved in pairs of floats
+constexpr int kSmallSolve = 256;               // widest system of the blocked solve
 // The fp32 factorisation's relative error grows with cond(X^T X + lambda I) times in 2^-24;
 // systems whose pivots show a condition number above this (cond >= (max L_ii / min L_ii)^2)
-// are factored again in double.
+// are solved again in pairs of floats.
 constexpr float kSmallSolveMaxCond = 1e3f;
 
 struct FitRows {
@@ -185,16 +186,14 @@ __global__ void __launch_bounds__(kFitThreads) fit_rows_kernel(const __grid_cons
 // One CTA per group g = (j*Ht + h)*2 + kv.  G: fp32 X^T X [in][in]; C: fp32 X^T Y, column-major
 // [dt][in] (element (a, o) at o*in + a); A, Z: double scratch [in][in] and [in][dt].
 // W out: the group's [in][dt] block of W_K or W_V in the cache dtype.
-// only: NULL, or int[groups]: solve only the groups marked nonzero.
 template <typename T>
 __global__ void __launch_bounds__(kSolveThreads) fit_solve_kernel(const float* __restrict__ G,
                                                                   const float* __restrict__ C, double* A, double* Z,
                                                                   T* wk, T* wv, int in, int dt, double lambda,
-                                                                  unsigned* status, const int* only)
+                                                                  unsigned* status)
 {
     __shared__ int bad;
     const int g = blockIdx.x;
-    if (only && !only[g]) return;
     double* a = A + (size_t)g * in * in;
     double* z = Z + (size_t)g * in * dt;
     const float* gg = G + (size_t)g * in * in;
@@ -240,115 +239,6 @@ __global__ void __launch_bounds__(kSolveThreads) fit_solve_kernel(const float* _
     T* w = (g & 1) ? wv : wk;
     const size_t off = (size_t)(g >> 1) * in * dt;   // (j*Ht + h) block of [Lt][Ht][in][dt]
     for (int i = threadIdx.x; i < in * dt; i += blockDim.x) w[off + i] = from_f32<T>(bad ? 0.f : (float)z[i]);
-    if (bad && threadIdx.x == 0) set_status(status, kFitNotPosDef);
-}
-
-// in <= kSmallSolve: the factor lives in shared memory as fp32, packed lower triangle (row r at
-// r(r+1)/2), followed by `cols` columns of solutions [in][cols].  The sums X^T X are fp32 already,
-// so a float factorisation loses nothing against them; it removes the L2 round trips of the
-// double, global-memory kernel above.  One CTA per group.
-constexpr int kSmallSolve = 256;
-constexpr int kSmallSolveThreads = 512;
-constexpr int kSmallSolveSmem = 227 * 1024 - 2048;   // dynamic shared memory budget
-
-// redo: int[1 + groups]; a group whose factor shows a condition number above kSmallSolveMaxCond
-// writes no W, sets redo[1 + g] and counts itself in redo[0] (fit_solve_kernel then solves it in
-// double).
-template <typename T>
-__global__ void __launch_bounds__(kSmallSolveThreads) fit_solve_small_kernel(const float* __restrict__ G,
-                                                                             const float* __restrict__ C, T* wk,
-                                                                             T* wv, int in, int dt, int cols,
-                                                                             float lambda, unsigned* status, int* redo)
-{
-    extern __shared__ float Lp[];          // packed lower triangle, then the solution block
-    __shared__ float colk[kSmallSolve];    // column k of L below the diagonal
-    __shared__ int bad, ill;
-    const int g = blockIdx.x;
-    const float* gg = G + (size_t)g * in * in;
-    const float* cc = C + (size_t)g * in * dt;
-    auto at = [](int r, int c) { return r * (r + 1) / 2 + c; };
-    float* zs = Lp + at(in, 0);            // [in][cols]
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarps = blockDim.x >> 5;
-    if (threadIdx.x == 0) bad = 0;
-    for (int r = warp; r < in; r += nwarps)
-        for (int c = lane; c <= r; c += 32) Lp[at(r, c)] = gg[(size_t)r * in + c] + (r == c ? lambda : 0.f);
-    __syncthreads();
-    // right-looking Cholesky: Lp = L with L L^T = X^T X + lambda I
-    for (int k = 0; k < in; ++k) {
-        if (threadIdx.x == 0) {
-            float d = Lp[at(k, k)];
-            if (!(d > 0.f)) { bad = 1; d = 1.f; }
-            Lp[at(k, k)] = sqrtf(d);
-        }
-        __syncthreads();
-        const float dk = Lp[at(k, k)];
-        for (int r = k + 1 + threadIdx.x; r < in; r += blockDim.x) {
-            const float v = Lp[at(r, k)] / dk;
-            Lp[at(r, k)] = v;
-            colk[r] = v;
-        }
-        __syncthreads();
-        for (int r = k + 1 + warp; r < in; r += nwarps) {
-            const float lr = colk[r];
-            for (int c = k + 1 + lane; c <= r; c += 32) Lp[at(r, c)] -= lr * colk[c];
-        }
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) {
-        float dmin = Lp[0], dmax = Lp[0];
-        for (int k = 1; k < in; ++k) {
-            const float d = Lp[at(k, k)];
-            dmin = fminf(dmin, d);
-            dmax = fmaxf(dmax, d);
-        }
-        const float ratio = dmax / dmin;
-        ill = !bad && ratio * ratio > kSmallSolveMaxCond;
-        if (ill) {
-            redo[1 + g] = 1;
-            atomicAdd(&redo[0], 1);
-        }
-    }
-    __syncthreads();
-    if (ill) return;
-    T* w = (g & 1) ? wv : wk;
-    const size_t off = (size_t)(g >> 1) * in * dt;
-    for (int o0 = 0; o0 < dt; o0 += cols) {
-        const int nc = min(cols, dt - o0);
-        // one thread per output column: L u = c, then L^T w = u, four independent partial sums
-        for (int o = threadIdx.x; o < nc; o += blockDim.x) {
-            for (int r = 0; r < in; ++r) {
-                const float* lr = Lp + at(r, 0);
-                float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
-                int k = 0;
-                for (; k + 3 < r; k += 4) {
-                    s0 = fmaf(lr[k], zs[(k + 0) * cols + o], s0);
-                    s1 = fmaf(lr[k + 1], zs[(k + 1) * cols + o], s1);
-                    s2 = fmaf(lr[k + 2], zs[(k + 2) * cols + o], s2);
-                    s3 = fmaf(lr[k + 3], zs[(k + 3) * cols + o], s3);
-                }
-                for (; k < r; ++k) s0 = fmaf(lr[k], zs[k * cols + o], s0);
-                zs[r * cols + o] = (cc[(size_t)(o0 + o) * in + r] - ((s0 + s1) + (s2 + s3))) / lr[r];
-            }
-            for (int r = in - 1; r >= 0; --r) {
-                float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
-                int k = r + 1;
-                for (; k + 3 < in; k += 4) {
-                    s0 = fmaf(Lp[at(k, r)], zs[k * cols + o], s0);
-                    s1 = fmaf(Lp[at(k + 1, r)], zs[(k + 1) * cols + o], s1);
-                    s2 = fmaf(Lp[at(k + 2, r)], zs[(k + 2) * cols + o], s2);
-                    s3 = fmaf(Lp[at(k + 3, r)], zs[(k + 3) * cols + o], s3);
-                }
-                for (; k < in; ++k) s0 = fmaf(Lp[at(k, r)], zs[k * cols + o], s0);
-                zs[r * cols + o] = (zs[r * cols + o] - ((s0 + s1) + (s2 + s3))) / Lp[at(r, r)];
-            }
-        }
-        __syncthreads();
-        for (int i = threadIdx.x; i < in * nc; i += blockDim.x) {
-            const int r = i / nc, o = i - r * nc;
-            w[off + (size_t)r * dt + o0 + o] = from_f32<T>(bad ? 0.f : zs[r * cols + o]);
-        }
-        __syncthreads();
-    }
     if (bad && threadIdx.x == 0) set_status(status, kFitNotPosDef);
 }
 
@@ -1024,16 +914,6 @@ __global__ void __launch_bounds__(gram_threads(DIRECT), 1) fit_gram_tc_kernel(co
     }
 }
 
-
-// solution columns per block for the small solve, and its dynamic shared memory
-int small_solve_cols(int in, int dt)
-{
-    const int tri = in * (in + 1) / 2;
-    const int cols = (kSmallSolveSmem / 4 - tri) / in;
-    return cols < dt ? cols : dt;
-}
-size_t small_solve_smem(int in, int cols) { return ((size_t)in * (in + 1) / 2 + (size_t)in * cols) * sizeof(float); }
-
 }  // namespace
 }  // namespace kvx
 
@@ -1041,7 +921,10 @@ using namespace kvx;
 
 struct kvx_fitter {
     Geometry geo;
-    int* redo = nullptr;                  // [1 + groups]: systems the fp32 solve hands to the double one
+    int* redo = nullptr;                  // [1 + groups], behind the status word: how many systems the fp32
+                                          // solve leaves to the pair solve, and each group's flag
+    float* factor = nullptr;              // blocks of the fp32 factors (in <= kSmallSolve)
+    float* factor_pair = nullptr;         // of the pair factors, once a solve has needed them
     int device = 0, num_sms = 0;
     int groups = 0, chunk = 0;
     int tc = 0;                           // Gram sums by fit_gram_tc_kernel (no row workspace)
@@ -1070,7 +953,8 @@ static void free_fitter(kvx_fitter* f)
 {
     if (!f) return;
     if (f->rows) cudaFree(f->rows);
-    if (f->redo) cudaFree(f->redo);
+    if (f->factor) cudaFree(f->factor);
+    if (f->factor_pair) cudaFree(f->factor_pair);
     if (f->sums) cudaFree(f->sums);
     if (f->rope) cudaFree(f->rope);
     if (f->status) cudaFree(f->status);
@@ -1082,6 +966,11 @@ static size_t sums_floats(const kvx_fitter* f)
 {
     const size_t in = f->geo.in_dim, dt = f->geo.desc.dst.head_dim;
     return (size_t)f->groups * in * (in + dt);
+}
+
+template <class S> static size_t factor_bytes(const kvx_fitter* f)
+{
+    return (size_t)f->groups * solve_blocks(f->geo.in_dim) * Blocks<S>::SZ * sizeof(float);
 }
 
 extern "C" KVX_API kvx_status kvx_fit_create(const kvx_translator_desc* desc, double lambda, int32_t chunk_tokens,
@@ -1125,12 +1014,14 @@ extern "C" KVX_API kvx_status kvx_fit_create(const kvx_translator_desc* desc, do
     }
     if ((f->rows_bytes && cudaMalloc(&f->rows, f->rows_bytes) != cudaSuccess) ||
         cudaMalloc(&f->sums, sums_floats(f) * sizeof(float)) != cudaSuccess ||
-        cudaMalloc(&f->rope, rope_bytes) != cudaSuccess || cudaMalloc(&f->status, sizeof(unsigned)) != cudaSuccess ||
-        cudaMalloc(&f->redo, sizeof(int) * (1 + (size_t)f->groups)) != cudaSuccess) {
+        cudaMalloc(&f->rope, rope_bytes) != cudaSuccess ||
+        cudaMalloc(&f->status, sizeof(int) * (2 + (size_t)f->groups)) != cudaSuccess ||
+        (in <= (size_t)kSmallSolve && cudaMalloc(&f->factor, factor_bytes<F32>(f)) != cudaSuccess)) {
         const size_t rb = f->rows_bytes;
         free_fitter(f);
         return fit_fail(KVX_ERR_OOM, "fit_create: device allocation (%zu bytes of rows)", rb);
     }
+    f->redo = (int*)f->status + 1;
     if ((ce = cudaMemcpy(f->rope, f->geo.turns, rope_bytes, cudaMemcpyHostToDevice)) != cudaSuccess ||
         (ce = cudaMemset(f->sums, 0, sums_floats(f) * sizeof(float))) != cudaSuccess ||
         (ce = cudaMemset(f->status, 0, sizeof(unsigned))) != cudaSuccess || (ce = cudaDeviceSynchronize()) != cudaSuccess) {
@@ -1266,44 +1157,62 @@ extern "C" KVX_API kvx_status kvx_fit_accumulate(kvx_fitter* f, const kvx_src_kv
     return KVX_OK;
 }
 
+// Factor and solve of every group (S = F32) or of the flagged ones (S = Pair).
+template <class S, typename T>
+static cudaError_t launch_solve(const kvx_fitter* f, float* factor, void* w_k, void* w_v, cudaStream_t s)
+{
+    const int in = f->geo.in_dim, dt = f->geo.desc.dst.head_dim;
+    const float* G = f->sums;
+    const float* C = f->sums + (size_t)f->groups * in * in;
+    fit_factor_kernel<S><<<f->groups, kFactorThreads, 0, s>>>(G, factor, in, f->lambda, kSmallSolveMaxCond,
+                                                              kFitNotPosDef, f->status, f->redo, f->redo + 1);
+    cudaError_t ce = cudaGetLastError();
+    if (ce != cudaSuccess) return ce;
+    const size_t smem = (size_t)kTrsmWarps * S::PL * in * kTrsmCols * sizeof(float);
+    if ((ce = smem_opt_in<fit_trsm_kernel<S, T>>((int)(kTrsmWarps * S::PL * kSmallSolve * kTrsmCols * sizeof(float)))) !=
+        cudaSuccess)
+        return ce;
+    const dim3 grid(f->groups, (dt / kTrsmCols + kTrsmWarps - 1) / kTrsmWarps);
+    fit_trsm_kernel<S, T><<<grid, kTrsmWarps * 32, smem, s>>>(C, factor, (T*)w_k, (T*)w_v, in, dt, f->redo + 1);
+    return cudaGetLastError();
+}
+template <class S>
+static cudaError_t launch_solve(const kvx_fitter* f, float* factor, void* w_k, void* w_v, cudaStream_t s)
+{
+    return f->geo.desc.dtype == KVX_BF16 ? launch_solve<S, __nv_bfloat16>(f, factor, w_k, w_v, s)
+                                         : launch_solve<S, float>(f, factor, w_k, w_v, s);
+}
+
 extern "C" KVX_API kvx_status kvx_fit_solve(kvx_fitter* f, void* w_k, void* w_v, uint32_t* status_bits, void* stream)
 {
     if (!f || !w_k || !w_v) return fit_fail(KVX_ERR_INVALID_ARG, "fit_solve: NULL argument");
     const kvx_translator_desc& D = f->geo.desc;
     const int in = f->geo.in_dim, dt = D.dst.head_dim;
-    const bool bf = D.dtype == KVX_BF16;
     cudaStream_t s = (cudaStream_t)stream;
-    const float* G = f->sums;
-    const float* C = f->sums + (size_t)f->groups * in * in;
     cudaError_t ce = cudaSuccess;
-    int n_double = in <= kSmallSolve ? 0 : f->groups;   // systems for the double solve
+    unsigned bits[2] = {0, 0};   // status word, systems left to the pair solve
     if (in <= kSmallSolve) {
-        // fp32 factor and a block of solution columns in shared memory; ill-conditioned systems
-        // are marked for the double solve
-        const int cols = small_solve_cols(in, dt);
-        const int smem = (int)small_solve_smem(in, cols);
-        if ((ce = cudaMemsetAsync(f->redo, 0, sizeof(int) * (1 + (size_t)f->groups), s)) == cudaSuccess) {
-            if (bf) {
-                ce = cudaFuncSetAttribute(fit_solve_small_kernel<__nv_bfloat16>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-                if (ce == cudaSuccess)
-                    fit_solve_small_kernel<__nv_bfloat16><<<f->groups, kSmallSolveThreads, smem, s>>>(
-                        G, C, (__nv_bfloat16*)w_k, (__nv_bfloat16*)w_v, in, dt, cols, (float)f->lambda, f->status, f->redo);
-            } else {
-                ce = cudaFuncSetAttribute(fit_solve_small_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-                if (ce == cudaSuccess)
-                    fit_solve_small_kernel<float><<<f->groups, kSmallSolveThreads, smem, s>>>(
-                        G, C, (float*)w_k, (float*)w_v, in, dt, cols, (float)f->lambda, f->status, f->redo);
-            }
-        }
-        if (ce == cudaSuccess) ce = cudaGetLastError();
-        if (ce == cudaSuccess) ce = cudaMemcpyAsync(&n_double, f->redo, sizeof(int), cudaMemcpyDeviceToHost, s);
-        if (ce == cudaSuccess) ce = cudaStreamSynchronize(s);
+        if ((ce = cudaMemsetAsync(f->redo, 0, sizeof(int), s)) == cudaSuccess &&
+            (ce = launch_solve<F32>(f, f->factor, w_k, w_v, s)) == cudaSuccess &&
+            (ce = cudaMemcpyAsync(bits, f->status, sizeof bits, cudaMemcpyDeviceToHost, s)) == cudaSuccess)
+            ce = cudaStreamSynchronize(s);
         if (ce != cudaSuccess) return fit_fail(KVX_ERR_CUDA, "fit_solve: %s", cudaGetErrorString(ce));
-    }
-    bool redone = false;
-    if (n_double > 0) {
+        if (bits[1]) {
+            if (!f->factor_pair && cudaMalloc(&f->factor_pair, factor_bytes<Pair>(f)) != cudaSuccess) {
+                f->factor_pair = nullptr;
+                return fit_fail(KVX_ERR_OOM, "fit_solve: scratch allocation");
+            }
+            if ((ce = launch_solve<Pair>(f, f->factor_pair, w_k, w_v, s)) == cudaSuccess &&
+                (ce = cudaMemcpyAsync(bits, f->status, sizeof bits[0], cudaMemcpyDeviceToHost, s)) == cudaSuccess)
+                ce = cudaStreamSynchronize(s);
+            if (ce != cudaSuccess) return fit_fail(KVX_ERR_CUDA, "fit_solve: %s", cudaGetErrorString(ce));
+            bits[0] |= kFitSolvedDouble;
+        }
+    } else {
         // double scratch for the factorisation and the solutions: the row workspace when it is
         // large enough, else a temporary allocation (the solve is not on the translation path)
+        const float* G = f->sums;
+        const float* C = f->sums + (size_t)f->groups * in * in;
         const size_t need = (size_t)f->groups * in * (in + dt) * sizeof(double);
         double* scratch = nullptr;
         bool own = false;
@@ -1315,27 +1224,21 @@ extern "C" KVX_API kvx_status kvx_fit_solve(kvx_fitter* f, void* w_k, void* w_v,
         }
         double* A = scratch;
         double* Z = scratch + (size_t)f->groups * in * in;
-        const int* only = in <= kSmallSolve ? f->redo + 1 : nullptr;
-        if (bf)
-            fit_solve_kernel<__nv_bfloat16><<<f->groups, kSolveThreads, 0, s>>>(G, C, A, Z, (__nv_bfloat16*)w_k,
-                                                                                (__nv_bfloat16*)w_v, in, dt, f->lambda,
-                                                                                f->status, only);
+        if (D.dtype == KVX_BF16)
+            fit_solve_kernel<__nv_bfloat16><<<f->groups, kSolveThreads, 0, s>>>(
+                G, C, A, Z, (__nv_bfloat16*)w_k, (__nv_bfloat16*)w_v, in, dt, f->lambda, f->status);
         else
             fit_solve_kernel<float><<<f->groups, kSolveThreads, 0, s>>>(G, C, A, Z, (float*)w_k, (float*)w_v, in, dt,
-                                                                        f->lambda, f->status, only);
+                                                                        f->lambda, f->status);
         ce = cudaGetLastError();
+        if (ce == cudaSuccess) ce = cudaMemcpyAsync(bits, f->status, sizeof bits[0], cudaMemcpyDeviceToHost, s);
         if (ce == cudaSuccess) ce = cudaStreamSynchronize(s);
         if (own) cudaFree(scratch);
         if (ce != cudaSuccess) return fit_fail(KVX_ERR_CUDA, "fit_solve: %s", cudaGetErrorString(ce));
-        redone = in <= kSmallSolve;
     }
-    unsigned bits = 0;
-    if ((ce = cudaMemcpy(&bits, f->status, sizeof bits, cudaMemcpyDeviceToHost)) != cudaSuccess)
-        return fit_fail(KVX_ERR_CUDA, "fit_solve: %s", cudaGetErrorString(ce));
-    if (redone) bits |= kFitSolvedDouble;
-    if (status_bits) *status_bits = bits;
-    if (bits & kFitNotPosDef)
-        return fit_fail(KVX_ERR_DEVICE_STATUS, "fit_solve: a system was not positive definite (status 0x%x)", bits);
+    if (status_bits) *status_bits = bits[0];
+    if (bits[0] & kFitNotPosDef)
+        return fit_fail(KVX_ERR_DEVICE_STATUS, "fit_solve: a system was not positive definite (status 0x%x)", bits[0]);
     return KVX_OK;
 }
 

@@ -272,9 +272,9 @@ def test_fit_fp32_tiny_matches_oracle_tightly():
 def test_fit_ill_conditioned_calibration_matches_oracle():
     """A calibration set whose two source heads nearly coincide (head 1 = head 0 + 3e-3 noise):
     X^T X + lambda I has a condition number above 1e6, where an fp32 Cholesky factor loses most
-    of its digits.  The fitter sees it in the factor's pivots and factors those systems again in
-    double (status bit 0x40); W then matches the oracle's fp64 solution within the bound of the
-    fp32 sums and a double factorisation.  fp32 caches, so the rows carry no bf16 rounding."""
+    of its digits.  The fitter sees it in the factor's pivots and solves those systems again in
+    pairs of floats (status bit 0x40); W then matches the oracle's fp64 solution within the bound of
+    the fp32 sums and a double factorisation.  fp32 caches, so the rows carry no bf16 rounding."""
     spec = SPECS["tiny_fp32"]
     c = make_case(spec, [456])
     rng = np.random.default_rng(21)
@@ -298,6 +298,42 @@ def test_fit_ill_conditioned_calibration_matches_oracle():
     bk, bv = _elementwise_bound(c, tk, tv, lam, ok, ov, chol_u=2.0 ** -53)
     _assert_elementwise(gk, ok, bk, "ill-conditioned K")
     _assert_elementwise(gv, ov, bv, "ill-conditioned V")
+
+
+@pytest.mark.parametrize("spread", [False, True])
+@pytest.mark.parametrize("ds,kl,dt", [(64, 1, 64), (64, 3, 256), (256, 1, 128)])
+def test_blocked_solve_sizes_match_a_double_solve(ds, kl, dt, spread):
+    """One, six and eight 32-channel blocks against numpy in double, fp32 caches without rotation, so X
+    is the source rows.  spread: channel scales over two decades send every system to the pair solve.
+    A Cholesky solve is invariant to channel scaling, so the error of the rescaled W stays that of the
+    unscaled system: cond(X) ^ 2 < 16 at T = 4 in, times the fp32 sums' (T) and the factor's (4 in)
+    rounding errors."""
+    import torch
+
+    from paper_2608_30963_gb300 import synth
+    L, n_in = 2, ds * kl
+    T = 4 * n_in + 3
+    rng = np.random.default_rng(31)
+    scale = 10.0 ** (-2.0 * rng.random(n_in)) if spread else np.ones(n_in)
+    src = [[torch.from_numpy((rng.standard_normal((1, 1, T, ds)) * scale[(l % kl) * ds:][:ds]).astype(np.float32)).cuda()
+            for l in range(L * kl)] for _ in range(2)]
+    tgt = [[torch.from_numpy(rng.standard_normal((1, 1, T, dt)).astype(np.float32)).cuda() for _ in range(L)]
+           for _ in range(2)]
+    lmap = [[j * kl + k for k in range(kl)] for j in range(L)]
+    f = kvx.Fitter(synth.ModelGeom(L * kl, 1, ds, 0.0), synth.ModelGeom(L, 1, dt, 0.0), 0.0,
+                   layer_map=lmap if kl > 1 else [r[0] for r in lmap], dtype=kvx.KVX_FP32, layers_per_target=kl)
+    i32 = lambda x: torch.tensor(x, dtype=torch.int32, device="cuda")
+    f.accumulate(src[0], src[1], i32([T]), i32([0, T]), T, tgt[0], tgt[1])
+    w = [torch.zeros((L, 1, n_in, dt), device="cuda") for _ in range(2)]
+    bits = f.solve(w[0], w[1])
+    assert bits == (0x40 if spread else 0), hex(bits)
+    for kv in range(2):
+        for j in range(L):
+            X = np.concatenate([src[kv][l].cpu().numpy()[0, 0] for l in lmap[j]], axis=1).astype(np.float64)
+            Y = tgt[kv][j].cpu().numpy()[0, 0].astype(np.float64)
+            ref = np.linalg.lstsq(X, Y, rcond=None)[0] * scale[:, None]
+            got = w[kv][j, 0].cpu().numpy() * scale[:, None]
+            assert _rel(got, ref) <= 16 * (T + 4 * n_in) * 2.0 ** -24, (kv, j, _rel(got, ref))
 
 
 def test_fit_two_calls_chunked_and_paged_agree_with_one_call():
