@@ -516,3 +516,35 @@ def test_more_target_layers_than_the_identity_kernel_takes():
                               [40], False, None, False)
     c = make_case(spec, [40, 17])
     _full_compare(c, kvx.KVX_PATH_AUTO)
+
+
+@pytest.mark.parametrize("dtype", [kvx.KVX_FP32, kvx.KVX_BF16])
+@pytest.mark.parametrize("Hs,ds,Ht,dt", [(2, 64, 1, 64), (2, 128, 2, 128), (1, 64, 2, 256)])
+def test_cuda_core_tile_sizes_agree(Hs, ds, Ht, dt, dtype):
+    """A 40-layer translation of 200 tokens takes 64-token tiles, its first two layers alone 16-token
+    tiles (compared with the oracle elsewhere): every output is one accumulator over the inputs in the
+    same order, so the two agree bit for bit.  Spans of 1..3 rows, a ragged last tile in both."""
+    L, T = 40, 200
+    rng = np.random.default_rng(5)
+    hi = np.cumsum(rng.choice([1, 2, 3], size=T))
+    lo = np.concatenate([[0], hi[:-1]])
+    S = int(hi[-1])
+    tdt = torch.float32 if dtype == kvx.KVX_FP32 else torch.bfloat16
+    i32 = lambda x: torch.tensor(np.asarray(x), dtype=torch.int32, device="cuda")
+    gen = torch.Generator(device="cuda").manual_seed(5)
+    rnd = lambda *sh: torch.randn(sh, device="cuda", generator=gen).to(tdt)
+    n_in = max(1, Hs // Ht) * ds
+    src = [[rnd(1, Hs, S, ds) for _ in range(L)] for _ in range(2)]
+    w = [rnd(L, Ht, n_in, dt) for _ in range(2)]
+    outs = []
+    for n in (L, 2):
+        tr = kvx.Translator(synth.ModelGeom(L, Hs, ds, 1e4), synth.ModelGeom(n, Ht, dt, 1e6), w[0][:n], w[1][:n],
+                            layer_map=list(range(n)), dtype=dtype, path=kvx.KVX_PATH_SIMT)
+        dst = [[torch.full((1, Ht, T, dt), float("nan"), dtype=tdt, device="cuda") for _ in range(n)] for _ in range(2)]
+        tr.translate(src[0], src[1], i32([S]), i32([0, T]), T, dst[0], dst[1], span_lo=i32(lo), span_hi=i32(hi))
+        torch.cuda.synchronize()
+        outs.append(dst)
+    for kv in range(2):
+        for j in range(2):
+            assert not outs[0][kv][j].isnan().any()
+            assert torch.equal(outs[0][kv][j], outs[1][kv][j]), (kv, j)

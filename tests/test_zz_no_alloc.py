@@ -126,3 +126,31 @@ def test_static_entry_clears_its_status_and_rejects_oversize():
     with pytest.raises(kvx.KvxError) as e:
         kvx.kvx_translate_static(big, wk.data_ptr(), wv.data_ptr(), src, tgt, dst, stream, True)
     assert e.value.status == kvx.KVX_ERR_UNSUPPORTED
+
+
+def test_static_entry_takes_caches_that_start_between_16_byte_groups():
+    """The entry checks strides, not pointers: caches that start one element off a 16-byte group give
+    what aligned ones give, bit for bit."""
+    from gpu_harness import DeviceCase, to_dev
+    kvx.build()
+    c = make_case(synth.config_specs()["tiny_fp32"], [77])
+    g = DeviceCase(c, path=kvx.KVX_PATH_SIMT, paged=False)
+    wk, wv = to_dev(c.w_k, c.spec.dtype), to_dev(c.w_v, c.spec.dtype)
+    stream = torch.cuda.current_stream().cuda_stream
+
+    def off_by_one(t):
+        flat = torch.empty(t.numel() + 1, dtype=t.dtype, device="cuda")
+        return flat[1:].view(t.shape).copy_(t)
+
+    outs = []
+    for shift in (False, True):
+        if shift:
+            for name in ("src_k", "src_v", "dst_k", "dst_v"):
+                setattr(g, name, [off_by_one(t) if t is not None else None for t in getattr(g, name)])
+        for t in g.dst_k + g.dst_v:
+            t.fill_(float("nan"))
+        src, tgt, dst = _structs(g)
+        assert kvx.kvx_translate_static(g.tr.desc, wk.data_ptr(), wv.data_ptr(), src, tgt, dst, stream, True) == 0
+        outs.append([t.clone() for t in g.dst_k + g.dst_v])
+    for a, b in zip(*outs):
+        assert not a.isnan().any() and torch.equal(a, b)
