@@ -12,8 +12,8 @@
 // Section 5 (T_theta per layer and KV head).
 //
 // Bound: fp32 FMA issue (128 a clock and SM).  Each output is one accumulator in ascending input
-// order.  A thread per output channel with scalar reads of A and W measured 608 us for 1000 tokens of
-// 7B -> 1.5B shapes (3.7 G FMA).
+// order.  1000 tokens of 7B -> 1.5B shapes (3.7 G FMA): 211 us; 608 us with a thread per output channel
+// and scalar reads of A and W.
 #include "kvx_common.cuh"
 #include "kvx_kernels.h"
 
@@ -60,6 +60,15 @@ __device__ __forceinline__ void store4(__nv_bfloat16* p, float4 x)
     } else {
         p[0] = a.x; p[1] = a.y; p[2] = b.x; p[3] = b.y;
     }
+}
+// (c0, c1) += x (w0, w1): one packed instruction for two fp32 FMAs, each rounded as fmaf.  The packed
+// form halves the issue slots of the projection (236 to 211 us for the case above).
+__device__ __forceinline__ void fma2(float& c0, float& c1, float x, float w0, float w1)
+{
+    asm("{\n\t.reg .b64 a, b, c;\n\tmov.b64 a, {%2, %2};\n\tmov.b64 b, {%3, %4};\n\tmov.b64 c, {%0, %1};\n\t"
+        "fma.rn.f32x2 c, a, b, c;\n\tmov.b64 {%0, %1}, c;\n\t}"
+        : "+f"(c0), "+f"(c1)
+        : "f"(x), "f"(w0), "f"(w1));
 }
 // R(-theta) of a pair (lo, hi): lo cos + hi sin, hi cos - lo sin
 __device__ __forceinline__ void unrotate(float& lo, float& hi, float2 cs)
@@ -204,14 +213,10 @@ __global__ void __launch_bounds__(kSimtThreads) translate_simt_kernel(const __gr
 #pragma unroll
                 for (int u = 0; u < TR; ++u) {
                     const float x = k == 0 ? av[u].x : k == 1 ? av[u].y : k == 2 ? av[u].z : av[u].w;
-                    acc[u][0] = fmaf(x, wl.x, acc[u][0]);
-                    acc[u][1] = fmaf(x, wl.y, acc[u][1]);
-                    acc[u][2] = fmaf(x, wl.z, acc[u][2]);
-                    acc[u][3] = fmaf(x, wl.w, acc[u][3]);
-                    acc[u][4] = fmaf(x, wh.x, acc[u][4]);
-                    acc[u][5] = fmaf(x, wh.y, acc[u][5]);
-                    acc[u][6] = fmaf(x, wh.z, acc[u][6]);
-                    acc[u][7] = fmaf(x, wh.w, acc[u][7]);
+                    fma2(acc[u][0], acc[u][1], x, wl.x, wl.y);
+                    fma2(acc[u][2], acc[u][3], x, wl.z, wl.w);
+                    fma2(acc[u][4], acc[u][5], x, wh.x, wh.y);
+                    fma2(acc[u][6], acc[u][7], x, wh.z, wh.w);
                 }
             }
         }
@@ -303,22 +308,24 @@ template <typename T>
 cudaError_t launch_simt_t(const TranslateParams& P, bool vec, bool big, cudaStream_t stream)
 {
     if (simt_slots(P.dt) == 32)
-        return big ? launch_simt<T, 32, 4>(P, vec, stream) : launch_simt<T, 32, 1>(P, vec, stream);
-    return big ? launch_simt<T, 64, 8>(P, vec, stream) : launch_simt<T, 64, 2>(P, vec, stream);
+        return big ? launch_simt<T, 32, 2>(P, vec, stream) : launch_simt<T, 32, 1>(P, vec, stream);
+    return big ? launch_simt<T, 64, 4>(P, vec, stream) : launch_simt<T, 64, 2>(P, vec, stream);
 }
 }  // namespace
 
 size_t simt_smem_bytes(int in_dim, int dt)
 {
-    const size_t big = simt_smem(in_dim, simt_slots(dt), 64);
+    const size_t big = simt_smem(in_dim, simt_slots(dt), 32);
     return big <= (size_t)kSimtSmemMax ? big : simt_smem(in_dim, simt_slots(dt), 16);
 }
 
 cudaError_t launch_translate_simt(const TranslateParams& P, int dtype, cudaStream_t stream)
 {
-    // 64-token tiles where they give two CTAs an SM (152 SMs) and A fits shared memory, else 16
-    const long long tiles = (long long)((P.T_total + 63) / 64) * P.Ht * (P.dt / (2 * simt_slots(P.dt))) * P.Lt * 2;
-    const bool big = tiles >= 2 * 152 && simt_smem(P.in_dim, simt_slots(P.dt), 64) <= (size_t)kSimtSmemMax;
+    // 32-token tiles where they give two CTAs an SM (152 SMs) and A fits shared memory, else 16: four CTAs of
+    // 32 tokens an SM overlap their phases (211 us; two of 64 tokens and 128 threads 256, of 256 threads 227),
+    // and below two CTAs an SM the chain of one CTA counts
+    const long long tiles = (long long)((P.T_total + 31) / 32) * P.Ht * (P.dt / (2 * simt_slots(P.dt))) * P.Lt * 2;
+    const bool big = tiles >= 2 * 152 && simt_smem(P.in_dim, simt_slots(P.dt), 32) <= (size_t)kSimtSmemMax;
     // the strides are whole 16-byte groups; the caches of the allocation-free entry may start anywhere
     uintptr_t a = 0;
     for (int i = 0; i < P.Lt * P.kl; ++i) a |= (uintptr_t)P.src_k[i] | (uintptr_t)P.src_v[i];

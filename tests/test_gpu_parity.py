@@ -521,7 +521,7 @@ def test_more_target_layers_than_the_identity_kernel_takes():
 @pytest.mark.parametrize("dtype", [kvx.KVX_FP32, kvx.KVX_BF16])
 @pytest.mark.parametrize("Hs,ds,Ht,dt", [(2, 64, 1, 64), (2, 128, 2, 128), (1, 64, 2, 256)])
 def test_cuda_core_tile_sizes_agree(Hs, ds, Ht, dt, dtype):
-    """A 40-layer translation of 200 tokens takes 64-token tiles, its first two layers alone 16-token
+    """A 40-layer translation of 200 tokens takes 32-token tiles, its first two layers alone 16-token
     tiles (compared with the oracle elsewhere): every output is one accumulator over the inputs in the
     same order, so the two agree bit for bit.  Spans of 1..3 rows, a ragged last tile in both."""
     L, T = 40, 200
