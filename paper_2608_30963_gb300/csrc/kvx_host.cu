@@ -37,6 +37,7 @@ struct kvx_translator {
     // for up to kPlanTokens target tokens per launch (longer calls run in chunks)
     static constexpr int kPlanTokens = 1 << 16;
     void* plan = nullptr;
+    void* row_plan = nullptr;    // row plan of the row-gather span kernel, where the geometry takes it
     int last_launches = 0;       // kernel launches of the most recent kvx_translate
     int last_span_tokens = 0;    // target tokens of the most recent call if it ran the span kernel, else 0
     int dbg_stall_unit1 = 0;     // kvx_debug_stall_next_translate, for the next call only
@@ -127,6 +128,7 @@ static void free_translator(kvx_translator* t)
     if (t->rope) cudaFree(t->rope);
     if (t->status) cudaFree(t->status);
     if (t->plan) cudaFree(t->plan);
+    if (t->row_plan) cudaFree(t->row_plan);
     delete t;
 }
 
@@ -381,6 +383,12 @@ extern "C" KVX_API kvx_status kvx_translator_create(const kvx_translator_desc* d
         st = fail(KVX_ERR_OOM, "create: span plan allocation");
         goto err;
     }
+    if (t->path == KVX_PATH_TCGEN05 && rope_rot_dim(s) == s.head_dim && rope_rot_dim(d) == d.head_dim &&
+        rows_supported(t->in_dim, d.head_dim, s.head_dim, share_heads(t->dense, t->r, t->e, d.num_kv_heads)) &&
+        cudaMalloc(&t->row_plan, rows_plan_bytes(kvx_translator::kPlanTokens)) != cudaSuccess) {
+        st = fail(KVX_ERR_OOM, "create: span plan allocation");
+        goto err;
+    }
     if ((ce = cudaMemset(t->status, 0, sizeof(unsigned))) != cudaSuccess ||
         (ce = cudaDeviceSynchronize()) != cudaSuccess) {
         st = fail(KVX_ERR_CUDA, "create: %s", cudaGetErrorString(ce));
@@ -482,6 +490,10 @@ static kvx_status translate_impl(kvx_translator* tr, const kvx_src_kv* src, cons
             }
         ce = launch_translate_tc_aligned(P, maps, tr->host_turns, tr->num_sms, (cudaStream_t)stream);
         tr->last_launches = 1;
+    } else if (tr->row_plan && rows_offsets_fit(P)) {
+        ce = launch_translate_rows(P, tr->num_sms, tr->plan, tr->row_plan, kvx_translator::kPlanTokens,
+                                   (cudaStream_t)stream, &tr->last_launches);
+        tr->last_span_tokens = P.T_total;
     } else if (tr->path == KVX_PATH_TCGEN05) {
         ce = launch_translate_tc(P, tr->tc, tr->num_sms, tr->plan, kvx_translator::kPlanTokens, (cudaStream_t)stream,
                                  &tr->last_launches);

@@ -24,6 +24,8 @@ struct TcConfig {
     int smem_bytes;
     int threads;
     int ok;            // geometry supported
+    int hpu;           // target heads of one unit of the window kernel
+    int streamed;      // its weights stream in pieces (else one resident image per group)
 };
 // share: target heads that read the same input rows (share_heads); it decides how many heads
 // one unit of the span kernel covers and so the weight images' output split n_tile.
@@ -41,6 +43,15 @@ void tc_plan_layout(int T_total, int plan_tokens, int* nsub, int* ent_off);
 // target tokens; *launches receives the number of launches made.
 cudaError_t launch_translate_tc(const TranslateParams& P, const TcConfig& cfg, int num_sms, void* plan,
                                 int plan_tokens, cudaStream_t stream, int* launches);
+
+// spans over gathered source rows (kvx_tc_rows.cu): grouped inputs of up to 256 channels, whole-head
+// rotations.  Same chunks and launches as launch_translate_tc; it also leaves the window plan.
+bool rows_supported(int in_dim, int dt, int ds, int share);
+// one head's rows lie within 2^32 16-byte units, as the plan's row offsets count them
+bool rows_offsets_fit(const TranslateParams& P);
+size_t rows_plan_bytes(int tokens);
+cudaError_t launch_translate_rows(const TranslateParams& P, int num_sms, void* window_plan, void* plan, int plan_tokens,
+                                  cudaStream_t stream, int* launches);
 
 // identity-alignment tensor-core path (tensor-TMA fed)
 bool aligned_supported(int in_dim, int dt, int ds, int share, int Lt, int batch, int kl);

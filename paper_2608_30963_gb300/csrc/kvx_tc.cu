@@ -39,6 +39,7 @@
 
 #include "kvx_common.cuh"
 #include "kvx_kernels.h"
+#include "kvx_span_plan.cuh"
 #include "kvx_tc_common.cuh"
 
 namespace kvx {
@@ -76,14 +77,6 @@ constexpr int kBarSlotEmpty = kBarSlotFull + kNumSlots;
 constexpr int kBarPair = kBarSlotEmpty + kNumSlots;   // +quad*2+{0,1}: the two epilogue warps of a quadrant meet
 constexpr int kBarMmaDone = kBarPair + 8;             // after an abort: the issued MMAs have completed
 constexpr int kNumBars = kBarMmaDone + 1;
-
-// Span plan of one 32-token sub-tile, written by span_plan_kernel once per
-// translation and read by every (layer, head, K|V) group of the tile:
-//   header  {b0, c0, rows, 0}: the window of source rows [c0, c0 + rows) of sequence b0
-//   entries {w0, lo, hi, b} x 32, longest span first: w0 = window row of the span
-//           start (low 16 bits, signed; -1: read from global memory) | A row within
-//           the sub-tile << 16 (0xFFFF: token past the end); [lo, hi) the clamped
-//           source span of sequence b.
 
 struct SpanEnt {
     int stage_row;   // window row of the span start; < 0: rows are read from global memory
@@ -196,72 +189,6 @@ __device__ __forceinline__ int piece_group(const Unit& x, int p, int spu, int Ht
 {
     const int hh = p / spu, s = p - hh * spu;
     return ((x.j * Ht + x.h + hh) * 2 + x.kv) * n_split + x.nt + s;
-}
-
-// Sequence metadata view: shared-memory copies of seq_off / src_seq_len when the
-// batch is small enough, else the global arrays.
-struct SeqView {
-    const int* off;    // [batch+1]
-    const int* slen;   // [batch]
-    int batch;
-    __device__ __forceinline__ int find(int tp) const
-    {
-        int lo = 0, hi = batch - 1;
-        while (lo < hi) {
-            const int mid = (lo + hi + 1) >> 1;
-            if (off[mid] <= tp) lo = mid; else hi = mid - 1;
-        }
-        return lo;
-    }
-};
-
-// Span bounds of target token tp as given (loaded ahead of use; identity: unused).
-__device__ __forceinline__ int2 load_span(const TranslateParams& P, int tp)
-{
-    if (P.span_lo && tp < P.T_total) return make_int2(__ldg(&P.span_lo[tp]), __ldg(&P.span_hi[tp]));
-    return make_int2(0, 0);
-}
-
-// Source-side resolution of one target token (sequence, clamped span) from its
-// loaded span bounds.
-__device__ __forceinline__ void resolve_src(const TranslateParams& P, const SeqView& sv, int tp, int2 span, int& b,
-                                            int& lo, int& hi)
-{
-    b = sv.find(tp);
-    const int t = tp - sv.off[b];
-    int S = sv.slen[b];
-    if (S > P.src_max_seq || S < 0) {
-        set_status(P.status, KVX_DEV_SEQ_CLAMPED);
-        S = S < 0 ? 0 : P.src_max_seq;
-    }
-    if (P.span_lo) { lo = span.x; hi = span.y; }
-    else { lo = t; hi = t + 1; }
-    if (lo < 0 || hi > S || hi <= lo) {
-        set_status(P.status, KVX_DEV_SPAN_CLAMPED);
-        lo = lo < 0 ? 0 : (lo > S - 1 ? S - 1 : lo);
-        hi = hi > S ? S : hi;
-        if (hi <= lo) hi = lo + 1;
-        if (S == 0) { lo = 0; hi = 0; }
-    }
-}
-
-// Target-side resolution: output row offset (-1: not written) and RoPE position.
-__device__ __forceinline__ void resolve_dst(const TranslateParams& P, const SeqView& sv, int tp, long long& dst_off,
-                                            int& pt)
-{
-    const int b = sv.find(tp);
-    const int t = tp - sv.off[b];
-    const int p = P.tgt_pos ? __ldg(&P.tgt_pos[tp]) : t;
-    pt = P.rt.enabled ? clamp_pos(p, P.max_position, P.status) : 0;
-    if (!P.paged) {
-        if (t >= P.dst_max_seq) { set_status(P.status, KVX_DEV_SEQ_CLAMPED); dst_off = -1; }
-        else dst_off = (long long)b * P.db + (long long)t * P.dts;
-    } else {
-        const int pi = t / P.page_size;
-        const int page = pi < P.max_pages ? __ldg(&P.page_table[(size_t)b * P.max_pages + pi]) : -1;
-        if (page < 0 || page >= P.num_pages) { set_status(P.status, KVX_DEV_PAGE_INVALID); dst_off = -1; }
-        else dst_off = ((long long)page * P.page_size + (t % P.page_size)) * (long long)P.Ht * P.dt;
-    }
 }
 
 // (cos, sin) for PP consecutive frequencies i0.. at position p, from the
@@ -768,29 +695,8 @@ __global__ void __launch_bounds__(128) span_plan_kernel(const __grid_constant__ 
     const int tp = t_begin + sub * kSub + lane;
     const bool valid = tp < t_end;
     int b = -1, lo = 0, hi = 0;
-    if (valid) resolve_src(P, sv, tp, load_span(P, tp), b, lo, hi);
-    // valid tokens are a prefix of the sub-tile, so lane 0 opens the window
-    const int b0 = __shfl_sync(0xffffffffu, b, 0);
-    const int c0 = __shfl_sync(0xffffffffu, lo, 0);
-    const bool same = valid && b == b0;
-    const int hmax = __reduce_max_sync(0xffffffffu, same ? hi : INT_MIN);
-    int R = hmax == INT_MIN ? 0 : max(hmax - c0, 0);
-    R = min(R, cap_rows);
-    const bool inwin = same && lo >= c0 && hi <= c0 + R;
-    const int stage_row = inwin ? lo - c0 : -1;
-    // rank: longest span first (lengths above 3 share a bucket), then lane order;
-    // tokens past the end last
-    const int key = valid ? min(max(hi - lo, 0), 3) : -1;
-    int rank = 0;
-#pragma unroll
-    for (int k = 3; k >= -1; --k) {
-        const unsigned bal = __ballot_sync(0xffffffffu, key == k);
-        if (k > key) rank += __popc(bal);
-        else if (k == key) rank += __popc(bal & ((1u << lane) - 1u));
-    }
-    const int w0 = (int)(((unsigned)stage_row & 0xFFFFu) | ((valid ? (unsigned)lane : 0xFFFFu) << 16));
-    ent[(size_t)sub * kSub + rank] = make_int4(w0, lo, hi, b < 0 ? 0 : b);
-    if (lane == 0) hdr[sub] = make_int4(b0 < 0 ? 0 : b0, c0, R, 0);
+    if (valid) resolve_src<true>(P, sv, tp, load_span(P, tp), b, lo, hi);
+    write_window_plan(valid, b, lo, hi, sub, lane, cap_rows, hdr, ent);
 }
 
 // Weight images: for group g = ((j*Ht + h)*2 + kv)*n_split + nt, the B operand
@@ -895,7 +801,7 @@ bool tc_layout(int in_dim, int dt, int ds, int share, TcLaunch& L)
     // Window slots of 48 source rows: a 32-token sub-tile of spans averaging 1.3
     // tokens needs ~42; tokens whose rows fall past the cap are read from global
     // memory.  Two A slots when four window slots still fit, else one.
-    L.cap_rows = 48;
+    L.cap_rows = kWindowRows;
     L.slot_bytes = L.cap_rows * L.row_bytes;
     for (int n_a = kMaxA; n_a >= 1; --n_a) {
         unsigned off = 0;
@@ -933,11 +839,13 @@ bool tc_layout(int in_dim, int dt, int ds, int share, TcLaunch& L)
 TcConfig tc_config(int in_dim, int dt, int ds, int share)
 {
     TcLaunch L{};
-    TcConfig c{0, 0, 0, kThreads, 0};
+    TcConfig c{0, 0, 0, kThreads, 0, 1, 0};
     if (!tc_layout(in_dim, dt, ds, share, L)) return c;
     c.n_tile = L.n_tile;
     c.n_split = L.n_split;
     c.smem_bytes = kSmemMax;
+    c.hpu = L.hpu;
+    c.streamed = L.n_b > 1;
     c.ok = 1;
     return c;
 }
@@ -955,24 +863,6 @@ cudaError_t launch_tc_weight_relayout(const void* w_k, const void* w_v, void* im
     tc_weight_relayout_kernel<<<(unsigned)((total + threads - 1) / threads), threads, 0, stream>>>(
         (const __nv_bfloat16*)w_k, (const __nv_bfloat16*)w_v, (uint8_t*)image, Lt, Ht, in_dim, dt, n_tile, rhalf_t);
     return cudaGetLastError();
-}
-
-// programmatic stream serialization: see the kernels' griddepcontrol.wait
-template <typename K, typename... Args>
-static cudaError_t launch_pdl(K kernel, int grid, int threads, size_t smem, cudaStream_t stream, Args... args)
-{
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(grid);
-    cfg.blockDim = dim3(threads);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, args...);
-    return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 template <int DS, bool MULTI>

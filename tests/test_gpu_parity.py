@@ -548,3 +548,41 @@ def test_cuda_core_tile_sizes_agree(Hs, ds, Ht, dt, dtype):
         for j in range(2):
             assert not outs[0][kv][j].isnan().any()
             assert torch.equal(outs[0][kv][j], outs[1][kv][j]), (kv, j)
+
+
+@pytest.mark.parametrize("T", [1, 128, 259])
+@pytest.mark.parametrize("law", ["one", "two", "nine", "mixed"])
+@pytest.mark.parametrize("Hs,ds,Ht,dt", [(1, 64, 1, 64), (4, 64, 1, 128), (2, 128, 1, 64), (1, 128, 2, 256), (1, 256, 1, 128)])
+def test_gathered_rows_kernel_edges(Hs, ds, Ht, dt, law, T):
+    """The row-gather kernel against the CUDA-core kernel (itself held to the oracle above): one to four
+    source heads of every width, one token, whole and ragged tiles, two sequences of which the second has
+    no source tokens left of its spans, spans of one row, of two, of nine (more further rows than the side
+    buffer holds) and of 1..12 overlapping and descending, explicit source positions.  Both sum in fp32;
+    the row-gather kernel rounds its input rows to bf16 first, a relative 2^-9 each."""
+    rng = np.random.default_rng(17)
+    n = {"one": np.ones(T, int), "two": np.full(T, 2), "nine": np.full(T, 9), "mixed": rng.integers(1, 13, size=T)}[law]
+    S = 400
+    lo = rng.integers(0, S - 12, size=T) if law == "mixed" else np.minimum(np.cumsum(n) - n, S - 9)
+    i32 = lambda x: torch.tensor(np.asarray(x), dtype=torch.int32, device="cuda")
+    gen = torch.Generator(device="cuda").manual_seed(3)
+    rnd = lambda *sh: torch.randn(sh, device="cuda", generator=gen).to(torch.bfloat16)
+    L, n_in = 3, max(1, Hs // Ht) * ds
+    src = [[rnd(2, Hs, S, ds) for _ in range(L)] for _ in range(2)]
+    w = [rnd(L, Ht, n_in, dt) for _ in range(2)]
+    t0 = T - T // 3                      # the second sequence's tokens: its source is empty
+    pos = i32(rng.permutation(2 * S))
+    outs = []
+    for path in (kvx.KVX_PATH_AUTO, kvx.KVX_PATH_SIMT):
+        tr = kvx.Translator(synth.ModelGeom(L, Hs, ds, 1e4), synth.ModelGeom(L, Ht, dt, 1e6), w[0], w[1],
+                            layer_map=list(range(L)), path=path)
+        dst = [[torch.full((2, Ht, T, dt), float("nan"), dtype=torch.bfloat16, device="cuda") for _ in range(L)] for _ in range(2)]
+        tr.translate(src[0], src[1], i32([S, 0]), i32([0, t0, T]), T, dst[0], dst[1], span_lo=i32(lo), span_hi=i32(lo + n),
+                     src_pos=pos)
+        torch.cuda.synchronize()
+        outs.append(torch.stack([torch.stack(d) for d in dst]).double())
+    a, b = outs
+    assert torch.equal(a.isnan(), b.isnan())          # the same rows written
+    a, b = a.nan_to_num(), b.nan_to_num()
+    assert a[:, :, 1].abs().max() == 0 and b[:, :, 1].abs().max() == 0   # no source tokens: zero rows
+    for kv in range(2):
+        assert (a[kv] - b[kv]).norm() <= 2.0 ** -8 * 1.5 * b[kv].norm(), (kv, (a[kv] - b[kv]).norm() / b[kv].norm())
