@@ -775,7 +775,12 @@ cudaError_t launch_translate_tc_aligned(const TranslateParams& T, const void* co
     const int grid = (int)(UH < num_sms ? UH : num_sms);
     // V shares paired with the K shares by cost (kvx_schedule.h)
     P.use_vmap = grid <= kMaxVmap;
-    if (P.use_vmap) pair_v_shares(grid, UH, P.m_tiles_max, P.vmap);
+    // (two sorts of one entry a CTA: kept while the split stays the same, as it does from call to call)
+    static thread_local struct { int grid; long long UH; int m_tiles; } paired = {0, 0, 0};
+    if (P.use_vmap && (paired.grid != grid || paired.UH != UH || paired.m_tiles != P.m_tiles_max)) {
+        pair_v_shares(grid, UH, P.m_tiles_max, P.vmap);
+        paired = {grid, UH, P.m_tiles_max};
+    }
     // the diagnostics' and the thread-store instantiations only when they are asked for
     const int var = P.plain_stores ? 2 : (P.wait_ns != 0 || P.stall_unit1 != 0 ? 1 : 0);
     switch (T.ds * 4 + var) {
