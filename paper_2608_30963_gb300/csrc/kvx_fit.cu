@@ -1168,12 +1168,10 @@ static cudaError_t launch_solve(const kvx_fitter* f, float* factor, void* w_k, v
                                                               kFitNotPosDef, f->status, f->redo, f->redo + 1);
     cudaError_t ce = cudaGetLastError();
     if (ce != cudaSuccess) return ce;
-    const size_t smem = (size_t)kTrsmWarps * S::PL * in * kTrsmCols * sizeof(float);
-    if ((ce = smem_opt_in<fit_trsm_kernel<S, T>>((int)(kTrsmWarps * S::PL * kSmallSolve * kTrsmCols * sizeof(float)))) !=
-        cudaSuccess)
-        return ce;
-    const dim3 grid(f->groups, (dt / kTrsmCols + kTrsmWarps - 1) / kTrsmWarps);
-    fit_trsm_kernel<S, T><<<grid, kTrsmWarps * 32, smem, s>>>(C, factor, (T*)w_k, (T*)w_v, in, dt, f->redo + 1);
+    auto smem = [](int n) { return (kTrsmStages * Blocks<S>::SZ + kTrsmWarps * S::PL * n * kTrsmCols) * sizeof(float); };
+    if ((ce = smem_opt_in<fit_trsm_kernel<S, T>>((int)smem(kSmallSolve))) != cudaSuccess) return ce;
+    const dim3 grid(f->groups, dt / (kTrsmWarps * kTrsmCols));   // d_t is 64, 128 or 256
+    fit_trsm_kernel<S, T><<<grid, kTrsmWarps * 32, smem(in), s>>>(C, factor, (T*)w_k, (T*)w_v, in, dt, f->redo + 1);
     return cudaGetLastError();
 }
 template <class S>

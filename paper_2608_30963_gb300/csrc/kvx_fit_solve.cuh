@@ -2,19 +2,19 @@
 //
 // Every group g is a system (X^T X + lambda I) W = X^T Y of `in` unknowns (a multiple of 32) and
 // dt right-hand sides.  Two launches in 32 x 32 blocks:
-//   fit_factor_kernel  one CTA per group: L L^T = X^T X + lambda I, right-looking.  Per block column
-//                      one warp factors the diagonal block in registers, then one thread per row
-//                      below solves against it while one further warp runs the same recurrence on
-//                      the unit rows (the inverse of the diagonal block), then one warp per 32 x 32
-//                      block applies the rank-32 update (a 4 x 8 tile a lane).
+//   fit_factor_kernel  one CTA per group: L L^T = X^T X + lambda I, right-looking.  Per block column the
+//                      CTA factors the diagonal block in shared memory and inverts its factor in the
+//                      same 32 steps; then one warp per 32 x 32 block multiplies the blocks below by the
+//                      inverse and applies the rank-32 update (a 4 x 8 tile a lane).
 //   fit_trsm_kernel    one warp per 8 right-hand sides of a group: L U = C, then L^T W = U, left-looking
 //                      with the inverted diagonal blocks, so every step is a small matrix product.
-// The blocks of L live in global scratch (352 KB a group at in = 256, read through L1/L2); the
-// solutions of a warp live in shared memory.
+// The blocks of L live in global scratch (352 KB a group at in = 256); the solves pass them through
+// shared memory, three in flight, for the warps of a CTA together.
 //
-// Bound: the chain of block columns of one group (the factor) and FMA issue (the solves).  One thread
-// per matrix column of an unblocked factor, with three barriers a column, and one thread per right-hand
-// side spent 2.0 ms on 112 systems of 256 x 128.
+// Bound: the chain of block columns of one group (the factor) and FMA issue (the solves).  All loops
+// are kept rolled and small: with the diagonal block and the rows below it unrolled in registers,
+// instruction fetch was most of the factor's time.
+// @FIGURES@
 //
 // Arithmetic is a parameter.  F32: fp32, for systems the pivots show to be well conditioned.  Pair:
 // unevaluated sums h + l of two floats (about 48 bits), products exact by FMA (Dekker's two-product) and
@@ -29,7 +29,8 @@ namespace {
 
 constexpr int kSolveBlk = 32;
 constexpr int kFactorThreads = 256;
-constexpr int kTrsmWarps = 4;
+constexpr int kTrsmWarps = 8;
+constexpr int kTrsmStages = 3;  // blocks of L in shared memory
 constexpr int kTrsmCols = 8;    // right-hand sides per warp
 
 struct F32 {
@@ -43,9 +44,8 @@ struct F32 {
     __device__ F32 neg() const { return F32{-h}; }
     __device__ F32 add(float x) const { return F32{h + x}; }
     __device__ F32 root() const { return F32{sqrtf(h)}; }
-    __device__ F32 inverse() const { return *this; }                // div() takes what inverse() gives
-    __device__ F32 div(F32 d) const { return F32{h / d.h}; }
-    __device__ F32 shfl(int s) const { return F32{__shfl_sync(0xffffffffu, h, s)}; }
+    __device__ F32 inverse() const { return F32{1.f / h}; }
+    __device__ F32 times(F32 x) const { return F32{h * x.h}; }
     __device__ float value() const { return h; }
 };
 
@@ -101,19 +101,15 @@ struct Pair {
         y.norm();
         return y;
     }
-    __device__ Pair div(Pair inv) const   // *this times an inverse()
+    __device__ Pair times(Pair x) const
     {
-        const float p = __fmul_rn(h, inv.h);
-        float e = __fmaf_rn(h, inv.h, -p);
-        e = __fmaf_rn(h, inv.l, e);
-        e = __fmaf_rn(l, inv.h, e);
+        const float p = __fmul_rn(h, x.h);
+        float e = __fmaf_rn(h, x.h, -p);
+        e = __fmaf_rn(h, x.l, e);
+        e = __fmaf_rn(l, x.h, e);
         Pair y{p, e};
         y.norm();
         return y;
-    }
-    __device__ Pair shfl(int s) const
-    {
-        return Pair{__shfl_sync(0xffffffffu, h, s), __shfl_sync(0xffffffffu, l, s)};
     }
     __device__ float value() const { return h + l; }
 };
@@ -162,124 +158,150 @@ __device__ __forceinline__ void store4(float* p, const S (&x)[4])
 // *n_redo; the Pair pass (redo) works on the kSolveRedo groups only.
 constexpr int kSolveRedo = 1, kSolveBad = 2;
 
+// acc -= A B^T over one 32 x 32 block pair; a, b: this lane's first row and column of blocks stored
+// (r, p) at p * 32 + r.
 template <class S>
-__global__ void __launch_bounds__(kFactorThreads, 1) fit_factor_kernel(const float* G, float* scratch, int in, double lambda,
-                                                                    float max_cond, unsigned bad_bit, unsigned* status,
-                                                                    int* n_redo, int* flags)
+__device__ __forceinline__ void block_product(S (&acc)[8][4], const float* a, const float* b)
+{
+#pragma unroll 2
+    for (int p = 0; p < kSolveBlk; ++p) {
+        S x[4], y[2][4];
+        load4(a + p * kSolveBlk, x);
+        load4(b + p * kSolveBlk, y[0]);
+        load4(b + p * kSolveBlk + 4, y[1]);
+#pragma unroll
+        for (int c = 0; c < 8; ++c)
+#pragma unroll
+            for (int r = 0; r < 4; ++r) acc[c][r].sub_mul(x[r], y[c >> 2][c & 3]);
+    }
+}
+
+template <class S>
+__global__ void __launch_bounds__(kFactorThreads, 2) fit_factor_kernel(const float* G, float* scratch, int in, double lambda,
+                                                                       float max_cond, unsigned bad_bit, unsigned* status,
+                                                                       int* n_redo, int* flags)
 {
     constexpr bool kRedo = S::PL == 2;
-    __shared__ float sD[S::PL * kPlane];        // the diagonal block's factor, (r, c) at c * 32 + r
-    __shared__ float sInv[S::PL * kSolveBlk];   // what div() by its diagonal takes
+    constexpr int kPitch = kSolveBlk + 1, kArea = kSolveBlk * kPitch, kWarps = kFactorThreads / 32;
+    // Diagonal block (r, c) at c * kPitch + r, the rows of its factor's inverse (r, c) at r * kPitch + c
+    // before their scaling, both in place; planes kArea apart.  First the warps' transposing tiles.
+    __shared__ float sh[kWarps * kArea];
     __shared__ float sPiv[256];
     __shared__ int sBad;
+    static_assert(2 * S::PL <= kWarps, "diagonal block and inverse fit the tiles");
+    float *sD = sh, *sE = sh + S::PL * kArea;
     const int g = blockIdx.x;
     if (kRedo && flags[g] != kSolveRedo) return;
     const int nb = in / kSolveBlk, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const Blocks<S> L{scratch + (size_t)g * solve_blocks(in) * Blocks<S>::SZ, nb};
     const float* gg = G + (size_t)g * in * in;
     if (threadIdx.x == 0) sBad = 0;
-    // lower blocks of X^T X + lambda I (only the lower triangle of the sums is kept)
-    for (int t = warp; t < nb * (nb + 1) / 2 * kSolveBlk; t += kFactorThreads / 32) {
-        const int b = t / kSolveBlk, r = t - b * kSolveBlk;
+    // lower blocks of X^T X (only the lower triangle of the sums is kept), transposed tile by tile
+    for (int t = warp; t < nb * (nb + 1) / 2; t += kWarps) {
         int i = 0;
-        while ((i + 1) * (i + 2) / 2 <= b) ++i;
-        const int j = b - i * (i + 1) / 2;
-        const bool diag = i == j && r == lane;
-        S v = S::make(gg[(size_t)(i * kSolveBlk + r) * in + j * kSolveBlk + lane]);
-        if (diag) v = v.add((float)lambda);
-        if (diag && kRedo) v = v.add((float)(lambda - (double)(float)lambda));
-        v.store(L.F(i, j) + lane * kSolveBlk + r, kPlane);
+        while ((i + 1) * (i + 2) / 2 <= t) ++i;
+        const int j = t - i * (i + 1) / 2;
+        float* tile = sh + warp * kArea;
+        __syncwarp();
+#pragma unroll 8
+        for (int r = 0; r < kSolveBlk; ++r)
+            tile[r * kPitch + lane] = gg[(size_t)(i * kSolveBlk + r) * in + j * kSolveBlk + lane];
+        __syncwarp();
+        float* f = L.F(i, j) + lane;
+#pragma unroll 8
+        for (int c = 0; c < kSolveBlk; ++c) S::make(tile[lane * kPitch + c]).store(f + c * kSolveBlk, kPlane);
     }
     __syncthreads();
 
+    const int dr = threadIdx.x >> 3, dc = threadIdx.x & 7;   // diagonal block: row, columns dc + 8 i
+    const int r0 = (lane & 7) * 4, c0 = (lane >> 3) * 8;     // block products: 4 rows x 8 columns a lane
     for (int k = 0; k < nb; ++k) {
-        if (warp == 0) {   // diagonal block: lane = row, its 32 entries in registers
-            S a[kSolveBlk];
-            float* d = L.F(k, k);
+        {   // diagonal block with lambda, and the unit matrix
+            const float* d = L.F(k, k);
 #pragma unroll
-            for (int c = 0; c < kSolveBlk; ++c) a[c] = S::load(d + c * kSolveBlk + lane, kPlane);
-            int bad = 0;
-#pragma unroll
-            for (int c = 0; c < kSolveBlk; ++c) {
-                S p = a[c].shfl(c);
-                if (!(p.value() > 0.f)) { bad = 1; p = S::make(1.f); }
-                const S l = p.root(), inv = l.inverse();
-                const S v = lane == c ? l : a[c].div(inv);
-                if (lane == 0) {
-                    inv.store(sInv + c, kSolveBlk);
-                    sPiv[k * kSolveBlk + c] = l.value();
+            for (int i = 0; i < 4; ++i) {
+                const int c = dc + 8 * i;
+                S v = S::load(d + c * kSolveBlk + dr, kPlane);
+                if (c == dr) {
+                    v = v.add((float)lambda);
+                    if (kRedo) v = v.add((float)(lambda - (double)(float)lambda));
                 }
-                v.store(sD + c * kSolveBlk + lane, kPlane);
-#pragma unroll
-                for (int q = c + 1; q < kSolveBlk; ++q) {
-                    a[q].sub_mul(v, v.shfl(q));
-                    if (q == c + 1) a[q].norm();
-                }
-            }
-            if (bad && lane == 0) sBad = 1;
-        }
-        __syncthreads();
-        // rows below, and the 32 unit rows whose solution is the inverse's columns
-        const int below = in - (k + 1) * kSolveBlk;
-        for (int t = threadIdx.x; t < below + kSolveBlk; t += kFactorThreads) {
-            const bool unit = t >= below;
-            const int row = unit ? t - below : t & 31, i = k + 1 + (t >> 5);
-            S x[kSolveBlk];
-            if (unit) {
-#pragma unroll
-                for (int c = 0; c < kSolveBlk; ++c) x[c] = S::make(c == row ? 1.f : 0.f);
-            } else {
-                const float* f = L.F(i, k) + row;
-#pragma unroll
-                for (int c = 0; c < kSolveBlk; ++c) x[c] = S::load(f + c * kSolveBlk, kPlane);
-            }
-#pragma unroll
-            for (int c = 0; c < kSolveBlk; ++c) {
-                x[c].norm();
-                x[c] = x[c].div(S::load(sInv + c, kSolveBlk));
-#pragma unroll
-                for (int q0 = 0; q0 < kSolveBlk; q0 += 4) {
-                    if (q0 + 3 <= c) continue;
-                    S l[4];
-                    load4(sD + c * kSolveBlk + q0, l);
-#pragma unroll
-                    for (int e = 0; e < 4; ++e)
-                        if (q0 + e > c) x[q0 + e].sub_mul(x[c], l[e]);
-                }
-            }
-            float* by_col = unit ? L.BI(k) : L.F(i, k);   // element c of this row at c * 32 + row
-            float* by_row = unit ? L.FI(k) : L.B(i, k);   // at row * 32 + c
-#pragma unroll
-            for (int c = 0; c < kSolveBlk; ++c) x[c].store(by_col + c * kSolveBlk + row, kPlane);
-#pragma unroll
-            for (int c0 = 0; c0 < kSolveBlk; c0 += 4) {
-                const S v[4] = {x[c0], x[c0 + 1], x[c0 + 2], x[c0 + 3]};
-                store4(by_row + row * kSolveBlk + c0, v);
+                v.store(sD + c * kPitch + dr, kArea);
+                S::make(c == dr ? 1.f : 0.f).store(sE + dr * kPitch + c, kArea);
             }
         }
         __syncthreads();
-        // rank-32 update of the blocks to the right: lane = 4 rows x 8 columns
-        const int m = nb - 1 - k, r0 = (lane & 7) * 4, c0 = (lane >> 3) * 8;
-        for (int t = warp; t < m * (m + 1) / 2; t += kFactorThreads / 32) {
+        // step p: column p of L = column p / sqrt(pivot), row p of the inverse likewise; later rows lose
+        // their multiples of both.  Column and row p are only read, the rest only written.
+#pragma unroll 1
+        for (int p = 0; p < kSolveBlk; ++p) {
+            S piv = S::load(sD + p * kPitch + p, kArea);
+            if (!(piv.value() > 0.f)) {
+                piv = S::make(1.f);
+                if (threadIdx.x == 0) sBad = 1;
+            }
+            const S root = piv.root(), inv = root.inverse();
+            if (threadIdx.x == 0) sPiv[k * kSolveBlk + p] = root.value();
+            if (dr > p) {
+                const S lr = S::load(sD + p * kPitch + dr, kArea).times(inv);
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const int c = dc + 8 * i;
+                    if (c > dr) continue;
+                    float* at = c > p ? sD + c * kPitch + dr : sE + dr * kPitch + c;
+                    const S other = S::load(c > p ? sD + p * kPitch + c : sE + p * kPitch + c, kArea).times(inv);
+                    S v = S::load(at, kArea);
+                    v.sub_mul(lr, other);
+                    v.norm();
+                    v.store(at, kArea);
+                }
+            }
+            __syncthreads();
+        }
+        // the inverse, its rows scaled: (r, c) both ways
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int c = dc + 8 * i;
+            S piv = S::load(sD + dr * kPitch + dr, kArea);
+            if (!(piv.value() > 0.f)) piv = S::make(1.f);
+            const S v = c <= dr ? S::load(sE + dr * kPitch + c, kArea).times(piv.root().inverse()) : S::make(0.f);
+            v.store(L.FI(k) + c * kSolveBlk + dr, kPlane);
+            v.store(L.BI(k) + dr * kSolveBlk + c, kPlane);
+        }
+        __syncthreads();
+        // blocks below: L(i, k) = A(i, k) inverse^T
+        for (int i = k + 1 + warp; i < nb; i += kWarps) {
+            S acc[8][4];
+#pragma unroll
+            for (int c = 0; c < 8; ++c)
+#pragma unroll
+                for (int r = 0; r < 4; ++r) acc[c][r] = S::make(0.f);
+            float *f = L.F(i, k), *bt = L.B(i, k);
+            block_product(acc, f + r0, L.FI(k) + c0);
+            __syncwarp();   // the block is overwritten
+#pragma unroll
+            for (int c = 0; c < 8; ++c) {
+#pragma unroll
+                for (int r = 0; r < 4; ++r) {
+                    acc[c][r].norm();
+                    acc[c][r] = acc[c][r].neg();
+                    acc[c][r].store(bt + (r0 + r) * kSolveBlk + c0 + c, kPlane);
+                }
+                store4(f + (c0 + c) * kSolveBlk + r0, acc[c]);
+            }
+        }
+        __syncthreads();
+        // rank-32 update of the blocks to the right
+        const int m = nb - 1 - k;
+        for (int t = warp; t < m * (m + 1) / 2; t += kWarps) {
             int i = 0;
             while ((i + 1) * (i + 2) / 2 <= t) ++i;
             const int j = t - i * (i + 1) / 2;
-            const float *fi = L.F(k + 1 + i, k) + r0, *fj = L.F(k + 1 + j, k) + c0;
             float* out = L.F(k + 1 + i, k + 1 + j) + c0 * kSolveBlk + r0;
             S acc[8][4];
 #pragma unroll
             for (int c = 0; c < 8; ++c) load4(out + c * kSolveBlk, acc[c]);
-#pragma unroll 4
-            for (int p = 0; p < kSolveBlk; ++p) {
-                S a[4], b[2][4];
-                load4(fi + p * kSolveBlk, a);
-                load4(fj + p * kSolveBlk, b[0]);
-                load4(fj + p * kSolveBlk + 4, b[1]);
-#pragma unroll
-                for (int c = 0; c < 8; ++c)
-#pragma unroll
-                    for (int r = 0; r < 4; ++r) acc[c][r].sub_mul(a[r], b[c >> 2][c & 3]);
-            }
+            block_product(acc, L.F(k + 1 + i, k) + r0, L.F(k + 1 + j, k) + c0);
 #pragma unroll
             for (int c = 0; c < 8; ++c) {
 #pragma unroll
@@ -314,13 +336,13 @@ __global__ void __launch_bounds__(kFactorThreads, 1) fit_factor_kernel(const flo
     }
 }
 
-// acc (rows 4 (lane % 8).. of a block, two columns) -= block . z, z[32][kTrsmCols] of one block row.
+// acc (rows 4 (lane % 8).. of a block row, two columns) -= block . z, z[32][kTrsmCols] of one block row.
 template <class S>
 __device__ __forceinline__ void trsm_step(S (&acc)[2][4], const float* block, const float* z, int zplane, int lane)
 {
     const float* a0 = block + (lane & 7) * 4;
     const float* z0 = z + (lane >> 3) * 2;
-#pragma unroll 8
+#pragma unroll 4
     for (int p = 0; p < kSolveBlk; ++p) {
         S a[4];
         load4(a0 + p * kSolveBlk, a);
@@ -333,18 +355,24 @@ __device__ __forceinline__ void trsm_step(S (&acc)[2][4], const float* block, co
     }
 }
 
-// C: X^T Y, column-major [dt][in]; W out in the cache dtype, [in][dt] per group.
-template <class S, typename T>
-__global__ void __launch_bounds__(kTrsmWarps * 32, 3) fit_trsm_kernel(const float* __restrict__ C,
-                                                                   const float* __restrict__ scratch, T* wk, T* wv,
-                                                                   int in, int dt, const int* __restrict__ flags)
+__device__ __forceinline__ void copy16(float* dst, const float* src)
 {
-    extern __shared__ float zs[];   // [warp][plane][in][kTrsmCols]
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
+}
+
+// C: X^T Y, column-major [dt][in]; W out in the cache dtype, [in][dt] per group.  dt is a multiple of the
+// CTA's kTrsmWarps * kTrsmCols columns.
+template <class S, typename T>
+__global__ void __launch_bounds__(kTrsmWarps * 32, 2) fit_trsm_kernel(const float* __restrict__ C,
+                                                                      const float* __restrict__ scratch, T* wk, T* wv,
+                                                                      int in, int dt, const int* __restrict__ flags)
+{
+    extern __shared__ float4 sm4[];   // [stage][block] | [warp][plane][in][kTrsmCols]
     constexpr bool kRedo = S::PL == 2;
+    constexpr int SZ = Blocks<S>::SZ;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int g = blockIdx.x, o0 = (blockIdx.y * kTrsmWarps + warp) * kTrsmCols;
     const int flag = flags[g];
-    if (o0 >= dt) return;
     T* w = ((g & 1) ? wv : wk) + (size_t)(g >> 1) * in * dt + o0;
     if (kRedo ? flag == 0 : flag == kSolveRedo) return;
     if (flag == kSolveBad) {
@@ -353,50 +381,75 @@ __global__ void __launch_bounds__(kTrsmWarps * 32, 3) fit_trsm_kernel(const floa
         return;
     }
     const int nb = in / kSolveBlk, zplane = in * kTrsmCols;
-    float* z = zs + (size_t)warp * S::PL * zplane;
-    const Blocks<S> L{const_cast<float*>(scratch) + (size_t)g * solve_blocks(in) * Blocks<S>::SZ, nb};
+    float* stage = reinterpret_cast<float*>(sm4);
+    float* z = stage + kTrsmStages * SZ + (size_t)warp * S::PL * zplane;
+    const Blocks<S> L{const_cast<float*>(scratch) + (size_t)g * solve_blocks(in) * SZ, nb};
+    // The blocks in the order both solves take them: per step s the s blocks of the row, then the inverse.
+    const int per_pass = nb * (nb + 1) / 2, total = 2 * per_pass;
+    int f_i = 0, f_pass = 0, f_s = 0, f_t = 0;   // next block to fetch
+    auto fetch = [&]() {
+        if (f_i < total) {
+            const int k = f_pass ? nb - 1 - f_s : f_s, j = f_pass ? nb - 1 - f_t : f_t;
+            const float* from = f_t == f_s ? (f_pass ? L.BI(k) : L.FI(k)) : (f_pass ? L.B(j, k) : L.F(k, j));
+            float* to = stage + (f_i % kTrsmStages) * SZ;
+            for (int e = threadIdx.x * 4; e < SZ; e += kTrsmWarps * 32 * 4) copy16(to + e, from + e);
+            ++f_i;
+            if (++f_t > f_s) {
+                f_t = 0;
+                if (++f_s == nb) { f_s = 0; ++f_pass; }
+            }
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");   // one group a call, empty ones at the end
+    };
+    for (int i = 0; i < kTrsmStages - 1; ++i) fetch();
     const float* cc = C + ((size_t)g * dt + o0) * in;
     for (int c = 0; c < kTrsmCols; ++c)
         for (int r = lane; r < in; r += 32) S::make(cc[(size_t)c * in + r]).store(z + r * kTrsmCols + c, zplane);
     __syncwarp();
     const int mine = (lane & 7) * 4 * kTrsmCols + (lane >> 3) * 2;   // this lane's first value of a block row
-    auto load_row = [&](int k, S (&acc)[2][4]) {
-#pragma unroll
-        for (int c = 0; c < 2; ++c)
-#pragma unroll
-            for (int r = 0; r < 4; ++r)
-                acc[c][r] = S::load(z + k * kSolveBlk * kTrsmCols + mine + r * kTrsmCols + c, zplane);
+    int n = 0;
+    // the next block: landed for every thread, the one before it free for the fetch after next
+    auto next_block = [&]() -> const float* {
+        asm volatile("cp.async.wait_group %0;" ::"n"(kTrsmStages - 2) : "memory");
+        __syncthreads();
+        fetch();
+        return stage + (n++ % kTrsmStages) * SZ;
     };
-    auto store_row = [&](int k, S (&acc)[2][4], bool neg) {
-        __syncwarp();   // every lane has read block row k
+    auto store_row = [&](float* row, S (&acc)[2][4], bool neg) {
+        __syncwarp();   // every lane has read the row
 #pragma unroll
         for (int c = 0; c < 2; ++c)
 #pragma unroll
             for (int r = 0; r < 4; ++r) {
                 acc[c][r].norm();
-                (neg ? acc[c][r].neg() : acc[c][r]).store(z + k * kSolveBlk * kTrsmCols + mine + r * kTrsmCols + c, zplane);
+                (neg ? acc[c][r].neg() : acc[c][r]).store(row + mine + r * kTrsmCols + c, zplane);
             }
         __syncwarp();
     };
-    auto row_of = [&](int k) { return z + k * kSolveBlk * kTrsmCols; };
-    S acc[2][4];
-    for (int pass = 0; pass < 2; ++pass) {   // L U = C, then L^T W = U
+#pragma unroll 1
+    for (int pass = 0; pass < 2; ++pass)   // L U = C, then L^T W = U
+#pragma unroll 1
         for (int s = 0; s < nb; ++s) {
-            const int k = pass ? nb - 1 - s : s;
-            load_row(k, acc);
-            for (int t = 0; t < s; ++t) {
-                const int j = pass ? nb - 1 - t : t;
-                trsm_step<S>(acc, pass ? L.B(j, k) : L.F(k, j), row_of(j), zplane, lane);
-            }
-            store_row(k, acc, false);
+            float* row = z + (pass ? nb - 1 - s : s) * kSolveBlk * kTrsmCols;
+            S acc[2][4];
 #pragma unroll
             for (int c = 0; c < 2; ++c)
 #pragma unroll
-                for (int r = 0; r < 4; ++r) acc[c][r] = S::make(0.f);
-            trsm_step<S>(acc, pass ? L.BI(k) : L.FI(k), row_of(k), zplane, lane);
-            store_row(k, acc, true);
+                for (int r = 0; r < 4; ++r) acc[c][r] = S::load(row + mine + r * kTrsmCols + c, zplane);
+#pragma unroll 1
+            for (int t = 0; t <= s; ++t) {
+                if (t == s) {   // the diagonal block: the row so far, times its inverse
+                    store_row(row, acc, false);
+#pragma unroll
+                    for (int c = 0; c < 2; ++c)
+#pragma unroll
+                        for (int r = 0; r < 4; ++r) acc[c][r] = S::make(0.f);
+                }
+                const float* zt = z + (pass ? nb - 1 - t : t) * kSolveBlk * kTrsmCols;
+                trsm_step<S>(acc, next_block(), zt, zplane, lane);
+            }
+            store_row(row, acc, true);
         }
-    }
     for (int r = lane; r < in; r += 32)
 #pragma unroll
         for (int c = 0; c < kTrsmCols; ++c)
