@@ -14,7 +14,9 @@
 // Bound: the chain of block columns of one group (the factor) and FMA issue (the solves).  All loops
 // are kept rolled and small: with the diagonal block and the rows below it unrolled in registers,
 // instruction fetch was most of the factor's time.
-// @FIGURES@
+// Measured, factor and solves: 112 systems of 256 x 128 in fp32 164 and 149 us (2.0 ms with an unblocked
+// factor and one thread per right-hand side); 208 systems of 128 x 256 in pairs 229 and 502 us, the
+// latter near the fp32 pipe's rate.
 //
 // Arithmetic is a parameter.  F32: fp32, for systems the pivots show to be well conditioned.  Pair:
 // unevaluated sums h + l of two floats (about 48 bits), products exact by FMA (Dekker's two-product) and
@@ -336,24 +338,135 @@ __global__ void __launch_bounds__(kFactorThreads, 2) fit_factor_kernel(const flo
     }
 }
 
-// acc (rows 4 (lane % 8).. of a block row, two columns) -= block . z, z[32][kTrsmCols] of one block row.
-template <class S>
-__device__ __forceinline__ void trsm_step(S (&acc)[2][4], const float* block, const float* z, int zplane, int lane)
+// Two floats in one register pair, and the packed instructions on them: each half rounds as its scalar
+// form does, at half the issue slots.
+struct F2 {
+    unsigned long long v;
+    __device__ static F2 make(float x, float y)
+    {
+        F2 r;
+        asm("mov.b64 %0, {%1, %2};" : "=l"(r.v) : "f"(x), "f"(y));
+        return r;
+    }
+    __device__ void get(float& x, float& y) const { asm("mov.b64 {%0, %1}, %2;" : "=f"(x), "=f"(y) : "l"(v)); }
+};
+__device__ __forceinline__ F2 add2(F2 a, F2 b)
 {
-    const float* a0 = block + (lane & 7) * 4;
-    const float* z0 = z + (lane >> 3) * 2;
-#pragma unroll 4
-    for (int p = 0; p < kSolveBlk; ++p) {
-        S a[4];
-        load4(a0 + p * kSolveBlk, a);
+    F2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
+__device__ __forceinline__ F2 mul2(F2 a, F2 b)
+{
+    F2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
+__device__ __forceinline__ F2 fma2(F2 a, F2 b, F2 c)
+{
+    F2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r.v) : "l"(a.v), "l"(b.v), "l"(c.v));
+    return r;
+}
+
+// One row of a block row of the solutions, kTrsmCols columns: acc -= L[row][p] z[p], as F32 or Pair does it.
+template <class S> struct TrsmRow;
+template <> struct TrsmRow<F32> {
+    F2 h[kTrsmCols / 2];
+    __device__ void load(const float* z, int)
+    {
 #pragma unroll
-        for (int c = 0; c < 2; ++c) {
-            const S b = S::load(z0 + p * kTrsmCols + c, zplane);
-#pragma unroll
-            for (int r = 0; r < 4; ++r) acc[c][r].sub_mul(a[r], b);
+        for (int q = 0; q < kTrsmCols / 4; ++q) {
+            const float4 x = reinterpret_cast<const float4*>(z)[q];
+            h[2 * q] = F2::make(x.x, x.y);
+            h[2 * q + 1] = F2::make(x.z, x.w);
         }
     }
-}
+    __device__ void zero()
+    {
+#pragma unroll
+        for (int c = 0; c < kTrsmCols / 2; ++c) h[c].v = 0;
+    }
+    __device__ void sub_mul(const float* l, const float* z, int)
+    {
+        const F2 a = F2::make(-*l, -*l);
+#pragma unroll
+        for (int c = 0; c < kTrsmCols / 4; ++c) {
+            const float4 b = reinterpret_cast<const float4*>(z)[c];
+            h[2 * c] = fma2(a, F2::make(b.x, b.y), h[2 * c]);
+            h[2 * c + 1] = fma2(a, F2::make(b.z, b.w), h[2 * c + 1]);
+        }
+    }
+    __device__ void store(float* z, int, bool neg) const
+    {
+        const float f = neg ? -1.f : 1.f;
+#pragma unroll
+        for (int q = 0; q < kTrsmCols / 4; ++q) {
+            float4 x;
+            h[2 * q].get(x.x, x.y);
+            h[2 * q + 1].get(x.z, x.w);
+            reinterpret_cast<float4*>(z)[q] = make_float4(f * x.x, f * x.y, f * x.z, f * x.w);
+        }
+    }
+};
+template <> struct TrsmRow<Pair> {
+    F2 h[kTrsmCols / 2], l[kTrsmCols / 2];
+    __device__ void load(const float* z, int plane)
+    {
+#pragma unroll
+        for (int q = 0; q < kTrsmCols / 4; ++q) {
+            const float4 x = reinterpret_cast<const float4*>(z)[q], y = reinterpret_cast<const float4*>(z + plane)[q];
+            h[2 * q] = F2::make(x.x, x.y);
+            h[2 * q + 1] = F2::make(x.z, x.w);
+            l[2 * q] = F2::make(y.x, y.y);
+            l[2 * q + 1] = F2::make(y.z, y.w);
+        }
+    }
+    __device__ void zero()
+    {
+#pragma unroll
+        for (int c = 0; c < kTrsmCols / 2; ++c) h[c].v = l[c].v = 0;
+    }
+    __device__ void sub_mul(const float* lp, const float* z, int plane)
+    {
+        const F2 lh = F2::make(lp[0], lp[0]), ah = F2::make(-lp[0], -lp[0]), al = F2::make(-lp[kPlane], -lp[kPlane]);
+        const F2 minus = F2::make(-1.f, -1.f);
+        auto sub2 = [&](F2 a, F2 b) { return fma2(b, minus, a); };   // a - b, rounded once
+#pragma unroll
+        for (int q = 0; q < kTrsmCols / 4; ++q) {
+            const float4 zh = reinterpret_cast<const float4*>(z)[q], zl = reinterpret_cast<const float4*>(z + plane)[q];
+            const F2 bh[2] = {F2::make(zh.x, zh.y), F2::make(zh.z, zh.w)}, bl[2] = {F2::make(zl.x, zl.y), F2::make(zl.z, zl.w)};
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                const int c = 2 * q + u;
+                // Pair::sub_mul: the product p and its error, the cross terms, Knuth's two-sum (np = -p)
+                const F2 np = mul2(lh, bh[u]);
+                const F2 e = fma2(al, bh[u], fma2(ah, bl[u], fma2(ah, bh[u], np)));
+                const F2 s = sub2(h[c], np), bb = sub2(s, h[c]);
+                const F2 t = sub2(sub2(h[c], sub2(s, bb)), add2(np, bb));
+                h[c] = s;
+                l[c] = add2(l[c], add2(t, e));
+            }
+        }
+    }
+    __device__ void store(float* z, int plane, bool neg) const
+    {
+        const float f = neg ? -1.f : 1.f;
+#pragma unroll
+        for (int q = 0; q < kTrsmCols / 4; ++q) {
+            Pair x[4];
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                h[2 * q + u].get(x[2 * u].h, x[2 * u + 1].h);
+                l[2 * q + u].get(x[2 * u].l, x[2 * u + 1].l);
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u) x[u].norm();
+            reinterpret_cast<float4*>(z)[q] = make_float4(f * x[0].h, f * x[1].h, f * x[2].h, f * x[3].h);
+            reinterpret_cast<float4*>(z + plane)[q] = make_float4(f * x[0].l, f * x[1].l, f * x[2].l, f * x[3].l);
+        }
+    }
+};
 
 __device__ __forceinline__ void copy16(float* dst, const float* src)
 {
@@ -406,7 +519,6 @@ __global__ void __launch_bounds__(kTrsmWarps * 32, 2) fit_trsm_kernel(const floa
     for (int c = 0; c < kTrsmCols; ++c)
         for (int r = lane; r < in; r += 32) S::make(cc[(size_t)c * in + r]).store(z + r * kTrsmCols + c, zplane);
     __syncwarp();
-    const int mine = (lane & 7) * 4 * kTrsmCols + (lane >> 3) * 2;   // this lane's first value of a block row
     int n = 0;
     // the next block: landed for every thread, the one before it free for the fetch after next
     auto next_block = [&]() -> const float* {
@@ -415,40 +527,27 @@ __global__ void __launch_bounds__(kTrsmWarps * 32, 2) fit_trsm_kernel(const floa
         fetch();
         return stage + (n++ % kTrsmStages) * SZ;
     };
-    auto store_row = [&](float* row, S (&acc)[2][4], bool neg) {
-        __syncwarp();   // every lane has read the row
-#pragma unroll
-        for (int c = 0; c < 2; ++c)
-#pragma unroll
-            for (int r = 0; r < 4; ++r) {
-                acc[c][r].norm();
-                (neg ? acc[c][r].neg() : acc[c][r]).store(row + mine + r * kTrsmCols + c, zplane);
-            }
-        __syncwarp();
-    };
 #pragma unroll 1
     for (int pass = 0; pass < 2; ++pass)   // L U = C, then L^T W = U
 #pragma unroll 1
         for (int s = 0; s < nb; ++s) {
-            float* row = z + (pass ? nb - 1 - s : s) * kSolveBlk * kTrsmCols;
-            S acc[2][4];
-#pragma unroll
-            for (int c = 0; c < 2; ++c)
-#pragma unroll
-                for (int r = 0; r < 4; ++r) acc[c][r] = S::load(row + mine + r * kTrsmCols + c, zplane);
+            float* mine = z + ((pass ? nb - 1 - s : s) * kSolveBlk + lane) * kTrsmCols;   // lane = row
+            TrsmRow<S> acc;
+            acc.load(mine, zplane);
 #pragma unroll 1
             for (int t = 0; t <= s; ++t) {
                 if (t == s) {   // the diagonal block: the row so far, times its inverse
-                    store_row(row, acc, false);
-#pragma unroll
-                    for (int c = 0; c < 2; ++c)
-#pragma unroll
-                        for (int r = 0; r < 4; ++r) acc[c][r] = S::make(0.f);
+                    acc.store(mine, zplane, false);
+                    acc.zero();
                 }
                 const float* zt = z + (pass ? nb - 1 - t : t) * kSolveBlk * kTrsmCols;
-                trsm_step<S>(acc, next_block(), zt, zplane, lane);
+                const float* l = next_block() + lane;   // the barrier also orders the warp's stores
+#pragma unroll 4
+                for (int p = 0; p < kSolveBlk; ++p) acc.sub_mul(l + p * kSolveBlk, zt + p * kTrsmCols, zplane);
             }
-            store_row(row, acc, true);
+            __syncwarp();   // every lane has read the row
+            acc.store(mine, zplane, true);
+            __syncwarp();
         }
     for (int r = lane; r < in; r += 32)
 #pragma unroll
