@@ -12,9 +12,16 @@
 // its tokens ordered by span length, longest first, so that the tokens with several rows are the first
 // `multi` rows of A.  Any spans will do: overlapping, repeated, descending, empty (a zero row).
 //
+// Inputs wider than 256 channels (several source layers, wide groups) are gathered and un-rotated 256
+// channels at a time (a K group) into the same accumulator; their weights do not stay but stream a K-block
+// at a time through a ring, in the MMA's order.  Groups of two source layers, 70B -> 7B shapes, 8192
+// tokens: 1092 us, 1339 in the window kernel.  Units of several heads (the dense form) stay there: with
+// four heads' weights to stream per K-block the ring's 64 KB do not cover the L2's latency (1294 against
+// 896 us).
+//
 // Persistent, one CTA per SM.  Work unit = (target layer j, target head h, K|V, output split nt, tile):
-//   warp 0         MMA: TMEM allocation, the group's B image (kept across its tiles), tcgen05.mma per
-//                  K-block (64 channels), commits
+//   warp 0         MMA: TMEM allocation, the group's B image (kept across its tiles, or streamed),
+//                  tcgen05.mma per K-block (64 channels), commits
 //   warps 1-2      gather: 64 rows each, into a ring of K-block slots
 //   warp 3         side buffer: the further rows of the tile's spans
 //   warps 4-11     epilogue: TMEM -> target RoPE -> bf16 -> cache (bulk row stores); two warps per lane
@@ -44,10 +51,11 @@ constexpr int kXfWarp0 = kEpiWarp0 + kNumEpiWarps;
 constexpr int kNumXfWarps = 8;
 constexpr int kThreads = (kXfWarp0 + kNumXfWarps) * 32;
 
-constexpr int kBarBFull = 0, kBarBEmpty = 1;
-constexpr int kBarDFull = 2;                        // +buf
-constexpr int kBarDEmpty = 4;                       // +buf
-constexpr int kBarFull = 6;                         // +slot: the gather's copies landed
+constexpr int kMaxB = 8;                            // weight ring slots (streamed)
+constexpr int kBarBFull = 0, kBarBEmpty = kMaxB;    // +weight slot
+constexpr int kBarDFull = 2 * kMaxB;                // +buf
+constexpr int kBarDEmpty = kBarDFull + 2;           // +buf
+constexpr int kBarFull = kBarDEmpty + 2;            // +slot: the gather's copies landed
 constexpr int kBarEmpty = kBarFull + kMaxSlots;     // +slot: MMA done with it
 // +(tile % nready): A is built (as many as tiles can lie between the prologue and the MMA)
 constexpr int kBarKReady = kBarEmpty + kMaxSlots;
@@ -78,7 +86,9 @@ struct TilePlan {
 };
 
 struct RowsLaunch {
-    int n_tile, n_split, in_dim, nblk, nslots, share;
+    int n_tile, n_split, nslots, share;
+    int nblk, kgs;         // K-blocks of a K group (at most 256 channels), K groups of an input row
+    int nb;                // weight ring slots, each a K-block; 0: the image stays resident
     int m_tiles;
     int side_rows;         // further rows the side buffer holds
     const TilePlan* tiles; // [tile]
@@ -92,39 +102,42 @@ struct RowsLaunch {
 // CTA walks its V share first, so that K tiles (un-rotated) and V tiles (streamed) run side by side.
 // share > 1: target heads that read the same source rows, walked by that many interleaved CTA sets,
 // so that partners read a tile's rows at about the same time and all but one find them in L2.
-struct RWalker {
-    // The walk, worked out once per CTA: units of the first share and in all, and where each share starts.
-    struct Start {
-        int n1, count;
-        int kv[2], j[2], h[2], nt[2], tile[2], h0[2];   // h0: this CTA's head among those that share rows
-        __device__ void init(const TranslateParams& P, const RowsLaunch& L)
-        {
-            const int E = L.share;
-            const long long UH = (long long)P.Lt * P.Ht * L.n_split * L.m_tiles / E;   // K (or V) units of one set
-            const int G = gridDim.x / E, c = blockIdx.x / E, rev = (int)(gridDim.x - 1 - blockIdx.x), cv = rev / E;
-            const int u0 = (int)((long long)c * UH / G), u1 = (int)((long long)(c + 1) * UH / G);
-            const int v0 = (int)((long long)cv * UH / G), v1 = (int)((long long)(cv + 1) * UH / G);
-            const bool v_first = (c & 1) == 0;
-            n1 = v_first ? v1 - v0 : u1 - u0;
-            count = (u1 - u0) + (v1 - v0);
-            for (int i = 0; i < 2; ++i) {
-                kv[i] = (i == 0) == v_first ? 1 : 0;
-                const int idx = kv[i] ? v0 : u0, hg = idx / L.m_tiles, jq = hg / L.n_split, HtE = P.Ht / E;
-                h0[i] = (kv[i] ? rev : (int)blockIdx.x) % E;
-                tile[i] = idx - hg * L.m_tiles;
-                nt[i] = hg % L.n_split;
-                h[i] = (jq % HtE) * E + h0[i];
-                j[i] = jq / HtE;
-            }
+// The walk, worked out once per CTA: units of the first share and in all, and where each share starts.
+struct RWalkStart {
+    int n1, count;
+    int kv[2], j[2], h[2], nt[2], tile[2], h0[2];   // h0: this CTA's head among those that share rows
+    __device__ void init(const TranslateParams& P, const RowsLaunch& L)
+    {
+        const int E = L.share;
+        const long long UH = (long long)P.Lt * P.Ht * L.n_split * L.m_tiles / E;   // K (or V) units of one set
+        const int G = gridDim.x / E, c = blockIdx.x / E, rev = (int)(gridDim.x - 1 - blockIdx.x), cv = rev / E;
+        const int u0 = (int)((long long)c * UH / G), u1 = (int)((long long)(c + 1) * UH / G);
+        const int v0 = (int)((long long)cv * UH / G), v1 = (int)((long long)(cv + 1) * UH / G);
+        const bool v_first = (c & 1) == 0;
+        n1 = v_first ? v1 - v0 : u1 - u0;
+        count = (u1 - u0) + (v1 - v0);
+        for (int i = 0; i < 2; ++i) {
+            kv[i] = (i == 0) == v_first ? 1 : 0;
+            const int idx = kv[i] ? v0 : u0, hg = idx / L.m_tiles, jq = hg / L.n_split, HtE = P.Ht / E;
+            h0[i] = (kv[i] ? rev : (int)blockIdx.x) % E;
+            tile[i] = idx - hg * L.m_tiles;
+            nt[i] = hg % L.n_split;
+            h[i] = (jq % HtE) * E + h0[i];
+            j[i] = jq / HtE;
         }
-    };
+    }
+};
+template <bool STREAM>
+struct RWalker {
     const TranslateParams& P;
     const RowsLaunch& L;
-    const Start& S;
+    const RWalkStart& S;
     int it, kv, j, h, nt, tile;
-    __device__ __forceinline__ RWalker(const TranslateParams& P_, const RowsLaunch& L_, const Start& S_) : P(P_), L(L_), S(S_)
+    int kg;   // K group
+    __device__ __forceinline__ RWalker(const TranslateParams& P_, const RowsLaunch& L_, const RWalkStart& S_) : P(P_), L(L_), S(S_)
     {
         it = 0;
+        kg = 0;
         share(S.n1 > 0 ? 0 : 1);
     }
     __device__ __forceinline__ void share(int i)
@@ -133,7 +146,16 @@ struct RWalker {
     }
     __device__ __forceinline__ int group() const { return ((j * P.Ht + h) * 2 + kv) * L.n_split + nt; }   // its B image
     __device__ __forceinline__ bool more() const { return it < S.count; }
+    // the next K group (of the unit, then of the next)
     __device__ __forceinline__ void next()
+    {
+        if (STREAM) {
+            if (++kg < L.kgs) return;
+            kg = 0;
+        }
+        next_unit();
+    }
+    __device__ __forceinline__ void next_unit()
     {
         ++it;
         if (it == S.n1) { share(1); return; }
@@ -145,8 +167,10 @@ struct RWalker {
             }
         }
     }
+    // tile of the next K group
+    __device__ __forceinline__ int next_tile() const { return STREAM && kg + 1 < L.kgs ? tile : next_unit_tile(); }
     // tile of the unit after this one (this one's after the last)
-    __device__ __forceinline__ int next_tile() const
+    __device__ __forceinline__ int next_unit_tile() const
     {
         if (it + 1 >= S.count) return tile;
         return it + 1 == S.n1 ? S.tile[1] : tile + 1 == L.m_tiles ? 0 : tile + 1;
@@ -209,8 +233,9 @@ __device__ __forceinline__ uint4 pack8(const float (&a)[8], float f)
     return make_uint4(pack_bf16(a[0] * f, a[1] * f), pack_bf16(a[2] * f, a[3] * f), pack_bf16(a[4] * f, a[5] * f),
                       pack_bf16(a[6] * f, a[7] * f));
 }
-// HS: half head_dim of the source (32, 64 or 128); HEADS: source heads of an input row
-template <int HS, int HEADS>
+// HS: half head_dim of the source (32, 64 or 128); HEADS: source heads of a K group; STREAM: several K groups,
+// weights streamed (else a resident image)
+template <int HS, int HEADS, bool STREAM>
 __global__ void __launch_bounds__(kThreads, 1)
 translate_rows_kernel(const __grid_constant__ TranslateParams P, const __grid_constant__ RowsLaunch L)
 {
@@ -224,7 +249,7 @@ translate_rows_kernel(const __grid_constant__ TranslateParams P, const __grid_co
     uint64_t* sBar = reinterpret_cast<uint64_t*>(smem + L.off_bar);
     volatile int* sAbort = reinterpret_cast<volatile int*>(smem + L.off_misc);
     uint32_t* sTmemBase = reinterpret_cast<uint32_t*>(smem + L.off_misc + 4);
-    RWalker::Start& sWalk = *reinterpret_cast<RWalker::Start*>(smem + L.off_misc + 16);
+    RWalkStart& sWalk = *reinterpret_cast<RWalkStart*>(smem + L.off_misc + 16);
     unsigned long long* sTurnS = reinterpret_cast<unsigned long long*>(smem + L.off_turns);
     unsigned long long* sTurnT = sTurnS + HS;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -234,8 +259,10 @@ translate_rows_kernel(const __grid_constant__ TranslateParams P, const __grid_co
     if (threadIdx.x == 32) sWalk.init(P, L);
     if (threadIdx.x == 0) {
         *sAbort = 0;
-        mbar_init(bar(kBarBFull), 1);
-        mbar_init(bar(kBarBEmpty), 1);
+        for (int i = 0; i < kMaxB; ++i) {
+            mbar_init(bar(kBarBFull + i), 1);
+            mbar_init(bar(kBarBEmpty + i), 1);
+        }
         for (int i = 0; i < 2; ++i) {
             mbar_init(bar(kBarDFull + i), 1);
             mbar_init(bar(kBarDEmpty + i), kNumEpiWarps);
@@ -276,12 +303,32 @@ translate_rows_kernel(const __grid_constant__ TranslateParams P, const __grid_co
     if (warp == kMmaWarp) {
         if (lane == 0) {
             const uint64_t pol_keep = policy_evict_last();
+            const uint32_t nb = STREAM ? (uint32_t)L.nb : 0u, kblock = (uint32_t)L.n_tile * 128;   // bytes of a K-block of weights
             int cur_g = -1;
-            uint32_t b_cnt = 0, tcount = 0, kr_idx = 0, kr_phase = 0;
+            uint32_t b_cnt = 0, tcount = 0, kr_idx = 0, kr_phase = 0;   // b_cnt: images or weight K-blocks loaded
             Slot sp{0, 0};
-            RWalker x(P, L, sWalk);
-            for (; x.more(); x.next()) {
-                if (x.group() != cur_g) {   // the group before has been multiplied when its last commit arrives
+            // streamed weights: the walk of the loads, nb - 1 K-blocks ahead of the MMAs
+            RWalker<STREAM> y(P, L, sWalk);
+            int y_kb = 0;
+            auto load_next = [&]() -> bool {
+                if (!y.more()) return true;
+                const uint32_t slot = b_cnt % nb;
+                if (!W.wait(bar(kBarBEmpty + slot), ((b_cnt / nb) & 1) ^ 1)) return false;
+                mbar_arrive_expect_tx(bar(kBarBFull + slot), kblock);
+                bulk_g2s(smem_u32(sB) + slot * kblock,
+                         (const uint8_t*)P.w + (size_t)y.group() * L.b_bytes + (size_t)(y.kg * L.nblk + y_kb) * kblock, kblock,
+                         bar(kBarBFull + slot), pol_keep);
+                ++b_cnt;
+                if (++y_kb == L.nblk) { y_kb = 0; y.next(); }
+                return true;
+            };
+            uint32_t b_use = 0;   // weight K-blocks multiplied
+            bool ok = true;
+            if (STREAM)
+                for (uint32_t i = 0; i + 1 < nb && ok; ++i) ok = load_next();
+            RWalker<STREAM> x(P, L, sWalk);
+            for (; x.more() && ok; x.next()) {
+                if (!STREAM && x.group() != cur_g) {   // the group before has been multiplied when its last commit arrives
                     if (!W.wait(bar(kBarBEmpty), (b_cnt & 1) ^ 1)) break;
                     mbar_arrive_expect_tx(bar(kBarBFull), L.b_bytes);
                     const uint8_t* img = (const uint8_t*)P.w + (size_t)x.group() * L.b_bytes;
@@ -293,31 +340,45 @@ translate_rows_kernel(const __grid_constant__ TranslateParams P, const __grid_co
                     cur_g = x.group();
                 }
                 const uint32_t buf = tcount & 1;
-                if (!W.wait(bar(kBarDEmpty + buf), ((tcount >> 1) & 1) ^ 1)) break;
-                const uint32_t d = tmem_base + buf * (uint32_t)L.n_tile, b0 = smem_u32(sB);
+                if ((!STREAM || x.kg == 0) && !W.wait(bar(kBarDEmpty + buf), ((tcount >> 1) & 1) ^ 1)) break;
                 if (!W.wait(bar(kBarKReady + kr_idx), kr_phase)) break;
                 if (++kr_idx == NKR) { kr_idx = 0; kr_phase ^= 1; }
                 tc_fence_after();
+                const uint32_t d = tmem_base + buf * (uint32_t)L.n_tile;
                 for (int kb = 0; kb < L.nblk; ++kb) {
-                    const uint32_t slot = sp.idx;
-                    const uint32_t a0 = smem_u32(sRing) + slot * kBlockBytes;
+                    const uint32_t a0 = smem_u32(sRing) + sp.idx * kBlockBytes;
+                    const uint32_t slot = STREAM ? b_use % nb : 0;
+                    const uint32_t b0 = smem_u32(sB) + (STREAM ? slot : (uint32_t)kb) * kblock;
+                    if (STREAM) {
+                        if (!W.wait(bar(kBarBFull + slot), (b_use / nb) & 1)) { ok = false; break; }
+                        tc_fence_after();
+                    }
 #pragma unroll
                     for (int kk = 0; kk < kBlockK / 16; ++kk)
-                        umma_bf16(d, sw128_desc(a0 + kk * 32), sw128_desc(b0 + kb * (L.n_tile * 128) + kk * 32), L.idesc,
-                                  (kb > 0 || kk > 0) ? 1u : 0u);
-                    umma_commit(bar(kBarEmpty + slot));
+                        umma_bf16(d, sw128_desc(a0 + kk * 32), sw128_desc(b0 + kk * 32), L.idesc,
+                                  ((STREAM && x.kg > 0) || kb > 0 || kk > 0) ? 1u : 0u);
+                    umma_commit(bar(kBarEmpty + sp.idx));
                     sp.adv(NS);
+                    if (STREAM) {
+                        umma_commit(bar(kBarBEmpty + slot));
+                        ++b_use;
+                        if (!load_next()) { ok = false; break; }
+                    }
                 }
-                umma_commit(bar(kBarDFull + buf));
-                if (x.last_of_group()) umma_commit(bar(kBarBEmpty));
-                ++tcount;
+                if (!ok) break;
+                if (!STREAM || x.kg + 1 == L.kgs) {
+                    umma_commit(bar(kBarDFull + buf));
+                    ++tcount;
+                }
+                if (!STREAM && x.last_of_group()) umma_commit(bar(kBarBEmpty));
             }
             if (*sAbort) {   // MMAs whose results nobody waited for must finish before TMEM is freed, copies land
                 umma_commit(bar(kBarMmaDone));
                 const unsigned long long t0 = globaltimer();
                 while (!mbar_try_wait(bar(kBarMmaDone), 0) && globaltimer() - t0 < W.limit_ns) {}
-                if (b_cnt)
-                    while (!mbar_try_wait(bar(kBarBFull), (b_cnt - 1) & 1) && globaltimer() - t0 < W.limit_ns) {}
+                const uint32_t n = STREAM ? nb : 1;
+                for (uint32_t c = b_cnt > n ? b_cnt - n : 0; c < b_cnt; ++c)
+                    while (!mbar_try_wait(bar(kBarBFull + c % n), (c / n) & 1) && globaltimer() - t0 < W.limit_ns) {}
             }
         }
         __syncwarp();
@@ -330,7 +391,7 @@ translate_rows_kernel(const __grid_constant__ TranslateParams P, const __grid_co
         uint8_t* srow = sStage + (size_t)m * L.stage_row_bytes;
         const uint32_t srow_u32 = smem_u32(srow);
         uint32_t tcount = 0;
-        RWalker x(P, L, sWalk);
+        RWalker<STREAM> x(P, L, sWalk);
         int n_nxt = -1;                     // the next unit's plan words, loaded a unit ahead
         int4 d_nxt = make_int4(0, 0, 0, 0);
         auto fetch = [&](int tile) {
@@ -339,14 +400,14 @@ translate_rows_kernel(const __grid_constant__ TranslateParams P, const __grid_co
             d_nxt = __ldg(&ent->dst);
         };
         if (x.more()) fetch(x.tile);
-        for (; x.more(); x.next()) {
-            const uint32_t buf = tcount & 1;
+        for (; x.more(); x.next_unit()) {
             const int4 ed = d_nxt;
             const bool valid = n_nxt >= 0;
-            fetch(x.next_tile());
+            fetch(x.next_unit_tile());
             const long long dst_off = (long long)(((unsigned long long)(unsigned)ed.y << 32) | (unsigned)ed.x);
             const int pt = ed.z;
             const bool rot = x.kv == 0 && P.rt.enabled;
+            const uint32_t buf = tcount & 1;
             if (!W.wait(bar(kBarDFull + buf), (tcount >> 1) & 1)) break;
             tc_fence_after();
             // the staging row is shared by the warps of this quadrant; the row's previous store must have
@@ -409,7 +470,7 @@ translate_rows_kernel(const __grid_constant__ TranslateParams P, const __grid_co
         };
         Slot sp{0, 0};
         uint32_t kr_idx = 0, ent_cnt = 0;
-        RWalker x(P, L, sWalk);
+        RWalker<STREAM> x(P, L, sWalk);
         int4 t_nxt = x.more() ? __ldg(&L.tiles[x.tile].count) : make_int4(0, 0, 0, 0);   // a unit ahead
         for (; x.more(); x.next()) {
             const bool rot = x.kv == 0 && P.rs.enabled;
@@ -426,7 +487,7 @@ translate_rows_kernel(const __grid_constant__ TranslateParams P, const __grid_co
                 const int k = s.w + o - 1;
                 if (k < L.side_rows) return reinterpret_cast<const uint4*>(sSide) + k * CPR + ch;
                 int slot, gq;
-                head_block(P, x.j, x.h, ch / (2 * CPH), slot, gq);
+                head_block(P, x.j, x.h, (STREAM ? x.kg * HEADS : 0) + ch / (2 * CPH), slot, gq);
                 return reinterpret_cast<const uint4*>((const __nv_bfloat16*)(x.kv ? P.src_v[slot] : P.src_k[slot]) +
                                                       (long long)gq * P.sh + (long long)(unsigned)s.x * 8 + o * P.ss +
                                                       (ch % (2 * CPH)) * 8);
@@ -549,7 +610,7 @@ translate_rows_kernel(const __grid_constant__ TranslateParams P, const __grid_co
             for (int i = 0; i < 2; ++i)
                 nxt[i] = __ldg(reinterpret_cast<const int2*>(&L.rows[(size_t)tile * kTileM + row0 + 32 * i + lane].src));
         };
-        RWalker x(P, L, sWalk);
+        RWalker<STREAM> x(P, L, sWalk);
         if (x.more()) fetch(x.tile);
         for (; x.more() && ok; x.next()) {
             cur[0] = nxt[0];
@@ -567,7 +628,7 @@ translate_rows_kernel(const __grid_constant__ TranslateParams P, const __grid_co
             for (int kb = 0; kb < L.nblk; ++kb) {
                 const int q = kb / (2 * HS / kBlockK), c0 = (kb - q * (2 * HS / kBlockK)) * kBlockK;
                 int src_slot, gq;
-                head_block(P, x.j, x.h, q, src_slot, gq);
+                head_block(P, x.j, x.h, (STREAM ? x.kg * HEADS : 0) + q, src_slot, gq);
                 const __nv_bfloat16* head = (const __nv_bfloat16*)(x.kv ? P.src_v[src_slot] : P.src_k[src_slot]) +
                                             (long long)gq * P.sh;
                 if (!W.wait(bar(kBarEmpty + sp.idx), sp.phase ^ 1)) { ok = false; break; }
@@ -600,7 +661,7 @@ translate_rows_kernel(const __grid_constant__ TranslateParams P, const __grid_co
 #pragma unroll
             for (int i = 0; i < kSideMax / 32; ++i) off_nxt[i] = __ldg(&L.tiles[tile].side[32 * i + lane]);
         };
-        RWalker x(P, L, sWalk);
+        RWalker<STREAM> x(P, L, sWalk);
         if (x.more()) fetch(x.tile);
         for (; x.more(); x.next(), ++cnt) {
             const int n = min(n_nxt, L.side_rows);
@@ -609,7 +670,7 @@ translate_rows_kernel(const __grid_constant__ TranslateParams P, const __grid_co
             for (int i = 0; i < kSideMax / 32; ++i) off[i] = off_nxt[i];
             fetch(x.next_tile());
             int slot, gq;
-            head_block(P, x.j, x.h, ch / CPH2, slot, gq);
+            head_block(P, x.j, x.h, (STREAM ? x.kg * HEADS : 0) + ch / CPH2, slot, gq);
             const uint4* from = reinterpret_cast<const uint4*>(
                 (const __nv_bfloat16*)(x.kv ? P.src_v[slot] : P.src_k[slot]) + (long long)gq * P.sh + (ch % CPH2) * 8);
             if (!W.wait(bar(kBarSideEmpty), (cnt & 1) ^ 1)) break;
@@ -706,12 +767,20 @@ __global__ void __launch_bounds__(kTileM) span_rows_kernel(const __grid_constant
 bool rows_layout(int in_dim, int dt, int ds, int share, RowsLaunch& L)
 {
     const TcConfig c = tc_config(in_dim, dt, ds, share);
-    if (!c.ok || in_dim > 256 || in_dim == 3 * ds || c.hpu != 1 || c.streamed) return false;
+    const int width = in_dim < 256 ? in_dim : 256;   // channels of a K group
+    if (!c.ok || c.hpu != 1 || in_dim % width || width == 3 * ds) return false;
     L.n_tile = c.n_tile;
     L.n_split = c.n_split;
-    L.in_dim = in_dim;
-    L.nblk = in_dim / kBlockK;
+    L.nblk = width / kBlockK;
+    L.kgs = in_dim / width;
     L.b_bytes = (unsigned)(in_dim * L.n_tile * 2);
+    // weights: the group's image where it fits, else a ring of K-blocks
+    constexpr unsigned kWeightBytes = 65536;
+    L.nb = 0;
+    if (c.streamed) {
+        L.nb = (int)(kWeightBytes / (unsigned)(L.n_tile * 128));
+        if (L.nb > kMaxB) L.nb = kMaxB;
+    }
     L.stage_row_bytes = (unsigned)(L.n_tile * 2 + 16);
     unsigned off = 0;
     auto take = [&](unsigned bytes, unsigned align) {
@@ -720,16 +789,16 @@ bool rows_layout(int in_dim, int dt, int ds, int share, RowsLaunch& L)
         off += bytes;
         return o;
     };
-    L.off_b = take(L.b_bytes, 1024);
+    L.off_b = take(L.nb ? (unsigned)(L.nb * L.n_tile * 128) : L.b_bytes, 1024);
     L.off_stage = take(kTileM * L.stage_row_bytes, 128);
     L.off_bar = take(kNumBars * 8, 8);
-    L.off_misc = take(16 + sizeof(RWalker::Start), 16);
+    L.off_misc = take(16 + sizeof(RWalkStart), 16);
     L.off_turns = take((unsigned)(ds / 2 + dt / 2) * 8, 16);
     L.off_ent = take(kEntTabs * kTileM * sizeof(int4), 16);
     L.off_ring = take(0, 1024);
     // K-block slots, of which a tile needs nblk, and the side buffer behind them: a tile of spans
     // averaging 1.3 rows has 38 further rows
-    const int avail = kSmemMax - 1024 - (int)L.off_ring, row = in_dim * 2;
+    const int avail = kSmemMax - 1024 - (int)L.off_ring, row = width * 2;
     int slots = (avail - 40 * row) / kBlockBytes;
     if (avail < 0 || slots < L.nblk) return false;
     L.nslots = slots < kMaxSlots ? slots : kMaxSlots;
@@ -743,12 +812,17 @@ bool rows_layout(int in_dim, int dt, int ds, int share, RowsLaunch& L)
     return cols <= 512;
 }
 
+template <int HS, int HEADS, bool STREAM>
+cudaError_t launch_rows_v(int grid, cudaStream_t stream, const TranslateParams& P, const RowsLaunch& L)
+{
+    const cudaError_t e = smem_opt_in<translate_rows_kernel<HS, HEADS, STREAM>>(kSmemMax);
+    if (e != cudaSuccess) return e;
+    return launch_pdl(translate_rows_kernel<HS, HEADS, STREAM>, grid, kThreads, kSmemMax, stream, P, L);
+}
 template <int HS, int HEADS>
 cudaError_t launch_rows(int grid, cudaStream_t stream, const TranslateParams& P, const RowsLaunch& L)
 {
-    const cudaError_t e = smem_opt_in<translate_rows_kernel<HS, HEADS>>(kSmemMax);
-    if (e != cudaSuccess) return e;
-    return launch_pdl(translate_rows_kernel<HS, HEADS>, grid, kThreads, kSmemMax, stream, P, L);
+    return L.nb ? launch_rows_v<HS, HEADS, true>(grid, stream, P, L) : launch_rows_v<HS, HEADS, false>(grid, stream, P, L);
 }
 
 }  // namespace
@@ -795,7 +869,7 @@ cudaError_t launch_translate_rows(const TranslateParams& P, int num_sms, void* w
         cudaError_t e = launch_pdl(span_rows_kernel, L.m_tiles, kTileM, 0, stream, P, t0, t1, kWindowRows, hdr, win, tiles, rows);
         if (e != cudaSuccess) return e;
         ++*launches;
-        switch (P.ds * 8 + P.in_dim / P.ds) {   // in <= 256, a multiple of ds
+        switch (P.ds * 8 + L.nblk * kBlockK / P.ds) {   // source heads of a K group
         case 64 * 8 + 1: e = launch_rows<32, 1>(grid, stream, P, L); break;
         case 64 * 8 + 2: e = launch_rows<32, 2>(grid, stream, P, L); break;
         case 64 * 8 + 4: e = launch_rows<32, 4>(grid, stream, P, L); break;

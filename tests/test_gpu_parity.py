@@ -552,10 +552,11 @@ def test_cuda_core_tile_sizes_agree(Hs, ds, Ht, dt, dtype):
 
 @pytest.mark.parametrize("T", [1, 128, 259])
 @pytest.mark.parametrize("law", ["one", "two", "nine", "mixed"])
-@pytest.mark.parametrize("Hs,ds,Ht,dt", [(1, 64, 1, 64), (4, 64, 1, 128), (2, 128, 1, 64), (1, 128, 2, 256), (1, 256, 1, 128)])
+@pytest.mark.parametrize("Hs,ds,Ht,dt", [(1, 64, 1, 64), (4, 64, 1, 128), (2, 128, 1, 64), (1, 128, 2, 256), (1, 256, 1, 128),
+                                         (4, 128, 1, 128), (4, 256, 1, 256)])
 def test_gathered_rows_kernel_edges(Hs, ds, Ht, dt, law, T):
     """The row-gather kernel against the CUDA-core kernel (itself held to the oracle above): one to four
-    source heads of every width, one token, whole and ragged tiles, two sequences of which the second has
+    source heads of every width (inputs of up to 256 channels, and two and four groups of 256), one token, whole and ragged tiles, two sequences of which the second has
     no source tokens left of its spans, spans of one row, of two, of nine (more further rows than the side
     buffer holds) and of 1..12 overlapping and descending, explicit source positions.  Both sum in fp32;
     the row-gather kernel rounds its input rows to bf16 first, a relative 2^-9 each."""
