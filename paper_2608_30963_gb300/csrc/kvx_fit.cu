@@ -183,7 +183,7 @@ __global__ void __launch_bounds__(kFitThreads) fit_rows_kernel(const __grid_cons
     }
 }
 
-// One CTA per group g = (j*Ht + h)*2 + kv.  G: fp32 X^T X [in][in]; C: fp32 X^T Y, column-major
+// One CTA per group g = (j*Ht + h)*2 + kv.  G: fp32 X^T X [in][in], element (r, c), c <= r, at c*in + r; C: fp32 X^T Y, column-major
 // [dt][in] (element (a, o) at o*in + a); A, Z: double scratch [in][in] and [in][dt].
 // W out: the group's [in][dt] block of W_K or W_V in the cache dtype.
 template <typename T>
@@ -201,7 +201,7 @@ __global__ void __launch_bounds__(kSolveThreads) fit_solve_kernel(const float* _
     if (threadIdx.x == 0) bad = 0;
     for (int i = threadIdx.x; i < in * in; i += blockDim.x) {
         const int r = i / in, c = i - r * in;
-        a[i] = c <= r ? (double)gg[i] + (r == c ? lambda : 0.0) : 0.0;
+        a[i] = c <= r ? (double)gg[(size_t)c * in + r] + (r == c ? lambda : 0.0) : 0.0;
     }
     __syncthreads();
     // right-looking Cholesky on the lower triangle: a = L L^T
@@ -244,7 +244,7 @@ __global__ void __launch_bounds__(kSolveThreads) fit_solve_kernel(const float* _
 
 // ------------------------------------------------------------------ Gram sums on the CUDA cores
 // One CTA per (group, 32-row block of X^T, 32-column block of the in + dt columns of Z = [X | Y]):
-// the block's sums over the pass's n tokens in fp32, added into G (X^T X, row-major [in][in]) or
+// the block's sums over the pass's n tokens in fp32, added into G (X^T X, [in][in], symmetric) or
 // C (X^T Y, column-major [dt][in]).  Each CTA owns its block, so plain read-modify-writes.
 template <typename T>
 __global__ void __launch_bounds__(256) fit_gram_simt_kernel(const T* __restrict__ X, const T* __restrict__ Y,
@@ -305,10 +305,14 @@ __global__ void __launch_bounds__(256) fit_gram_simt_kernel(const T* __restrict_
 //   MMA thread   M = 128 (the row block's channels as A), N over the needed columns (B, in
 //                pieces of <= 256), K = 16 tokens per instruction, into one fp32 TMEM
 //                accumulator that lives for the CTA's range of a unit.
-//   4 epilogue warps  add the accumulator into the fp32 sums (vector atomics for X^T X rows,
-//                coalesced atomics for X^T Y columns).
-// Units are (g, chunk of K-blocks, mb) with mb fastest; each CTA takes an equal contiguous
-// range of the (unit, K-block) space, so a range may start or end inside a unit.
+//   4 epilogue warps  add the accumulator into the fp32 sums, a column at a time (128 bytes an atomic
+//                instruction; 16-byte atomics along X^T X rows touched 32 lines each and held the
+//                accumulator, and with it the MMAs, longer: 199 against 190 us a 4096-token batch).
+// Units are (g, mb) with mb fastest.  Each CTA takes one contiguous range of the K groups' (unit, K-block)
+// space and one of the V groups', of equal cost (a block costs the rows it builds), so a range may start or
+// end inside a unit; every second CTA takes its V range first.  K blocks are un-rotated and V blocks only
+// copied: with one range over both, the CTAs that got K blocks ran on alone at the end (4096 tokens, 7B -> 1.5B
+// shapes: 206 us; 199 with two ranges, 190 with the flushes below).
 constexpr int kGramK = 64;
 constexpr int kGramMmaWarp = 0;
 constexpr int kGramEpiWarp0 = 1;
@@ -337,9 +341,7 @@ struct GramLaunch {
     int nrows;             // in + dt (rows of a full Z^T block)
     int mbs;               // row blocks of 128 input channels: in / 128
     int nkb;               // K-blocks of 64 tokens in the call
-    int kc;                // K-blocks per unit (a chunk); nkb % kc == 0
-    int nch;               // chunks: nkb / kc
-    int units;             // groups * nch * mbs
+    int units;             // groups * mbs
     int stages;            // Z^T block ring depth
     unsigned stage_bytes;  // nrows * 128
     int raw_slots;         // raw staging ring depth
@@ -348,7 +350,7 @@ struct GramLaunch {
     unsigned raw_bytes;    // one raw slot: token table, header, source window, target rows
     unsigned off_raw, off_bar;
     unsigned lbo, sbo;     // MN-major operand strides: between 64-channel blocks, between 8-token groups
-    float* G;              // [groups][in][in]
+    float* G;              // [groups][in][in], element (i, n) of X^T X at n * in + i
     float* C;              // [groups][dt][in]
 };
 
@@ -379,17 +381,49 @@ __device__ __forceinline__ uint32_t gram_chunk(int i, int c)
     return (uint32_t)((c >> 6) * (kGramK * 128) + (i >> 3) * 1024 + (i & 7) * 128 + ((((c >> 3) & 7) ^ (i & 7)) << 4));
 }
 
-// Unit u of the (g, chunk, mb) space and K-block index within the unit.
+// A CTA's blocks in order: n1 blocks from block a0 of the first kind's space (K or V groups), then those from
+// b0 of the other's.
 struct GramUnit {
     int g, mb, kb;   // kb: K-block of the call
 };
-__device__ __forceinline__ GramUnit gram_unit(const GramLaunch& L, int w)
-{
-    const int u = w / L.kc, kbi = w - u * L.kc;
-    const int mb = u % L.mbs, gc = u / L.mbs;
-    const int ch = gc % L.nch, g = gc / L.nch;
-    return GramUnit{g, mb, ch * L.kc + kbi};
-}
+struct GramRange {
+    int a0, b0, n1, n, kv1;   // kv1: K|V of the first n1 blocks
+    // first block of CTA c's share of one kind's space: rows built before it are c / grid of all
+    __device__ static int bound(const GramLaunch& L, int dt, int c, int grid)
+    {
+        long long per = 0;                           // rows built per K-block over a group's row blocks
+        for (int mb = 0; mb < L.mbs; ++mb) per += (mb + 1) * 128 + dt;
+        const long long total = (long long)(L.units / 2 / L.mbs) * L.nkb * per;
+        const long long at = c * total / grid, group = at / (L.nkb * per);
+        long long rest = at - group * L.nkb * per;
+        int mb = 0;
+        while (mb + 1 < L.mbs && rest >= (long long)L.nkb * ((mb + 1) * 128 + dt)) rest -= (long long)L.nkb * (++mb * 128 + dt);
+        return (int)((group * L.mbs + mb) * L.nkb + rest / ((mb + 1) * 128 + dt));
+    }
+    __device__ void init(const GramLaunch& L, int dt)
+    {
+        const int c = blockIdx.x, grid = gridDim.x, r = grid - 1 - c;
+        const int k0 = bound(L, dt, c, grid), k1 = bound(L, dt, c + 1, grid);
+        const int v0 = bound(L, dt, r, grid), v1 = bound(L, dt, r + 1, grid);
+        kv1 = c & 1 ? 0 : 1;
+        a0 = kv1 ? v0 : k0;
+        b0 = kv1 ? k0 : v0;
+        n1 = kv1 ? v1 - v0 : k1 - k0;
+        n = (k1 - k0) + (v1 - v0);
+    }
+    __device__ __forceinline__ GramUnit at(const GramLaunch& L, int i) const
+    {
+        const int w = i < n1 ? a0 + i : b0 + (i - n1), kv = i < n1 ? kv1 : kv1 ^ 1;
+        const int u = w / L.nkb, gp = u / L.mbs;
+        return GramUnit{gp * 2 + kv, u - gp * L.mbs, w - u * L.nkb};
+    }
+    // block i opens / closes an accumulator
+    __device__ __forceinline__ bool first(const GramUnit& x, int i) const { return i == 0 || i == n1 || x.kb == 0; }
+    __device__ __forceinline__ bool last(const GramLaunch& L, const GramUnit& x, int i) const
+    {
+        return i + 1 == n || i + 1 == n1 || x.kb + 1 == L.nkb;
+    }
+};
 
 // Channels [c_lo, +8) and [c_hi, +8) of token i, rounded to bf16, into the block.
 __device__ __forceinline__ void gram_put(uint8_t* st, int i, int c_lo, int c_hi, const float (&lo)[8], const float (&hi)[8])
@@ -440,8 +474,10 @@ __global__ void __launch_bounds__(gram_threads(DIRECT), 1) fit_gram_tc_kernel(co
     volatile int* sAbort = reinterpret_cast<volatile int*>(sBar + bDone + 1);
     uint32_t* sTmem = reinterpret_cast<uint32_t*>(sBar + bDone + 2);
     unsigned long long* sTurn = reinterpret_cast<unsigned long long*>(sBar + bDone + 4);   // source | target
+    GramRange* sRange = reinterpret_cast<GramRange*>(sTurn + (P.ds >> 1) + (P.dt >> 1));
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     auto bar = [&](int i) { return smem_u32(&sBar[i]); };
+    if (threadIdx.x == 32) sRange->init(L, P.dt);
     if (threadIdx.x == 0) {
         *sAbort = 0;
         for (int i = 0; i < L.stages; ++i) {
@@ -469,9 +505,7 @@ __global__ void __launch_bounds__(gram_threads(DIRECT), 1) fit_gram_tc_kernel(co
     tc_fence_after();
     const uint32_t tmem_base = *sTmem;
     const Waiter W{sAbort, P.status};
-    const long long total = (long long)L.units * L.kc;
-    const int w0 = (int)((long long)blockIdx.x * total / gridDim.x);
-    const int w1 = (int)((long long)(blockIdx.x + 1) * total / gridDim.x);
+    const GramRange R = *sRange;
     const int in = NHD * DS, dt = P.dt;
     constexpr int heads = NHD;
     auto tok_tab = [&](int r) { return reinterpret_cast<GramTok*>(sRaw + (size_t)r * L.raw_bytes); };
@@ -487,10 +521,9 @@ __global__ void __launch_bounds__(gram_threads(DIRECT), 1) fit_gram_tc_kernel(co
         if (lane == 0) {
             uint32_t it = 0, ucount = 0;
             bool issued = false;
-            for (int w = w0; w < w1; ++w, ++it) {
-                const GramUnit x = gram_unit(L, w);
-                const int kbi = w % L.kc;
-                const bool first = w == w0 || kbi == 0, last = w == w1 - 1 || kbi == L.kc - 1;
+            for (int i = 0; i < R.n; ++i, ++it) {
+                const GramUnit x = R.at(L, i);
+                const bool first = R.first(x, i), last = R.last(L, x, i);
                 const uint32_t s = it % (uint32_t)L.stages, ph = (it / (uint32_t)L.stages) & 1;
                 if (first && !W.wait(bar(bDEmpty), (ucount & 1) ^ 1)) break;
                 if (!W.wait(bar(bZFull + s), ph)) break;
@@ -532,30 +565,26 @@ __global__ void __launch_bounds__(gram_threads(DIRECT), 1) fit_gram_tc_kernel(co
         // ------------------------------------------------------------ epilogue: accumulator -> sums
         const int quad = warp & 3;
         uint32_t ucount = 0;
-        const int u_first = w0 / L.kc, u_last = w1 > w0 ? (w1 - 1) / L.kc : u_first - 1;
-        for (int u = u_first; u <= u_last; ++u, ++ucount) {
+        for (int i = 0; i < R.n; ++ucount) {
+            const GramUnit x = R.at(L, i);
+            // past the accumulator's blocks: to the end of its unit or of its range
+            i = min(i + L.nkb - x.kb, i < R.n1 ? R.n1 : R.n);
             if (!W.wait(bar(bDFull), ucount & 1)) break;
             tc_fence_after();
-            const GramUnit x = gram_unit(L, u * L.kc);
             const int nx = (x.mb + 1) * 128;
             const int row = x.mb * 128 + quad * 32 + lane;
-            float* grow = L.G + ((size_t)x.g * in + row) * in;
+            // column c of X^T X or X^T Y: the warp's 32 rows are neighbours in memory
+            float* gg = L.G + (size_t)x.g * in * in + row;
             float* cg = L.C + (size_t)x.g * dt * in + row;
             const uint32_t taddr = tmem_base + ((uint32_t)(quad * 32) << 16);
+#pragma unroll 1
             for (int c0 = 0; c0 < nx + dt; c0 += 32) {
                 uint32_t r[32];
                 tmem_ld32(taddr + c0, r);
                 tmem_ld_wait();
-                if (c0 < nx) {
+                float* to = c0 < nx ? gg + (size_t)c0 * in : cg + (size_t)(c0 - nx) * in;
 #pragma unroll
-                    for (int q = 0; q < 8; ++q)
-                        atomicAdd(reinterpret_cast<float4*>(grow + c0 + 4 * q),
-                                  make_float4(__uint_as_float(r[4 * q]), __uint_as_float(r[4 * q + 1]),
-                                              __uint_as_float(r[4 * q + 2]), __uint_as_float(r[4 * q + 3])));
-                } else {
-#pragma unroll
-                    for (int e = 0; e < 32; ++e) atomicAdd(cg + (size_t)(c0 - nx + e) * in, __uint_as_float(r[e]));
-                }
+                for (int e = 0; e < 32; ++e) atomicAdd(to + (size_t)e * in, __uint_as_float(r[e]));
             }
             tc_fence_before();
             __syncwarp();
@@ -566,8 +595,8 @@ __global__ void __launch_bounds__(gram_threads(DIRECT), 1) fit_gram_tc_kernel(co
         const uint64_t pol = policy_evict_last();   // the partner row block reads them again
         uint32_t it = 0, issued = 0;
         bool ok = true;
-        for (int w = w0; w < w1 && ok; ++w, ++it) {
-            const GramUnit x = gram_unit(L, w);
+        for (int i = 0; i < R.n && ok; ++i, ++it) {
+            const GramUnit x = R.at(L, i);
             const int kv = x.g & 1, jh = x.g >> 1, h = jh % P.Ht, j = jh / P.Ht;
             const uint32_t r = it % (uint32_t)L.raw_slots, ph = (it / (uint32_t)L.raw_slots) & 1;
             if (!W.wait(bar(bREmpty + r), ph ^ 1)) break;
@@ -575,7 +604,7 @@ __global__ void __launch_bounds__(gram_threads(DIRECT), 1) fit_gram_tc_kernel(co
             GramTok tk[2];
 #pragma unroll
             for (int u = 0; u < 2; ++u) {
-                const int i = lane + 32 * u, tp = x.kb * kGramK + i;
+                const int row = lane + 32 * u, tp = x.kb * kGramK + row;
                 tk[u] = GramTok{0, 0, 0, 0, -1, 0, 0};
                 if (tp < P.T_total) {
                     const TokenInfo ti = resolve_token(P, tp);
@@ -583,7 +612,7 @@ __global__ void __launch_bounds__(gram_threads(DIRECT), 1) fit_gram_tc_kernel(co
                     const int ps = DIRECT && ok && kv == 0 && P.rs.enabled ? src_pos_of(P, ti.b, ti.lo) : 0;
                     tk[u] = GramTok{ti.b, ti.lo, ti.hi, ti.pt, ti.dst_off, ok, ps};
                 }
-                tt[i] = tk[u];
+                tt[row] = tk[u];
             }
             if (DIRECT) {   // the prologue gathers the rows itself
                 __syncwarp();
@@ -667,8 +696,8 @@ __global__ void __launch_bounds__(gram_threads(DIRECT), 1) fit_gram_tc_kernel(co
         const unsigned long long* sTurnS = sTurn;
         const unsigned long long* sTurnT = sTurn + (P.ds >> 1);
         uint32_t it = (uint32_t)team;
-        for (int w = w0 + team; w < w1; w += kGramTeams, it += kGramTeams) {
-            const GramUnit x = gram_unit(L, w);
+        for (int blk = team; blk < R.n; blk += kGramTeams, it += kGramTeams) {
+            const GramUnit x = R.at(L, blk);
             const int kv = x.g & 1, jh = x.g >> 1, h = jh % P.Ht, j = jh / P.Ht;
             const int nh = min(heads, ((x.mb + 1) * 128 + DS - 1) / DS);
             const uint32_t s = it % (uint32_t)L.stages, ph = (it / (uint32_t)L.stages) & 1;
@@ -784,8 +813,8 @@ __global__ void __launch_bounds__(gram_threads(DIRECT), 1) fit_gram_tc_kernel(co
         const unsigned long long* sTurnS = sTurn;
         const unsigned long long* sTurnT = sTurn + (P.ds >> 1);
         uint32_t it = 0;
-        for (int w = w0; w < w1; ++w, ++it) {
-            const GramUnit x = gram_unit(L, w);
+        for (int blk = 0; blk < R.n; ++blk, ++it) {
+            const GramUnit x = R.at(L, blk);
             const int kv = x.g & 1, jh = x.g >> 1, h = jh % P.Ht, j = jh / P.Ht;
             // X head-blocks this row block needs: the rows [0, (mb+1)*128) of the lower triangle
             const int nh = min(heads, ((x.mb + 1) * 128 + DS - 1) / DS);
@@ -1075,13 +1104,11 @@ extern "C" KVX_API kvx_status kvx_fit_accumulate(kvx_fitter* f, const kvx_src_kv
         L.nrows = in + dt;
         L.mbs = in / 128;
         L.nkb = (tgt->total_tokens + kGramK - 1) / kGramK;
-        L.kc = L.nkb;   // one unit per (group, row block): one accumulator flush each
-        L.nch = L.nkb / L.kc;
-        L.units = f->groups * L.nch * L.mbs;
+        L.units = f->groups * L.mbs;
         L.stage_bytes = (unsigned)L.nrows * 128;
         L.src_row = (unsigned)ds * 2;   // rows as in the caches: whole windows move in one copy
         L.tgt_row = (unsigned)dt * 2;
-        const unsigned tail = 32 * 8 + (unsigned)(ds / 2 + dt / 2) * 8;   // barriers, flags, turns
+        const unsigned tail = 32 * 8 + (unsigned)(ds / 2 + dt / 2) * 8 + sizeof(GramRange);   // barriers, flags, turns, range
         // identity alignment: every span is one source row (or none), gathered by the prologue
         const bool direct = P.span_lo == nullptr;
         bool fits = false;
@@ -1114,7 +1141,7 @@ extern "C" KVX_API kvx_status kvx_fit_accumulate(kvx_fitter* f, const kvx_src_kv
         L.sbo = 1024;           // next 8-token atom row
         L.G = G;
         L.C = C;
-        const long long work = (long long)L.units * L.kc;
+        const long long work = (long long)L.units * L.nkb;
         const int grid = (int)(work < f->num_sms ? work : f->num_sms);
         const size_t smem = 1024 + (size_t)L.off_bar + tail;
         cudaError_t ce;

@@ -14,8 +14,8 @@
 // Bound: the chain of block columns of one group (the factor) and FMA issue (the solves).  All loops
 // are kept rolled and small: with the diagonal block and the rows below it unrolled in registers,
 // instruction fetch was most of the factor's time.
-// Measured, factor and solves: 112 systems of 256 x 128 in fp32 164 and 149 us (2.0 ms with an unblocked
-// factor and one thread per right-hand side); 208 systems of 128 x 256 in pairs 229 and 502 us, the
+// Measured, factor and solves: 112 systems of 256 x 128 in fp32 151 and 149 us (2.0 ms with an unblocked
+// factor and one thread per right-hand side); 208 systems of 128 x 256 in pairs 220 and 502 us, the
 // latter near the fp32 pipe's rate.
 //
 // Arithmetic is a parameter.  F32: fp32, for systems the pivots show to be well conditioned.  Pair:
@@ -186,11 +186,10 @@ __global__ void __launch_bounds__(kFactorThreads, 2) fit_factor_kernel(const flo
     constexpr bool kRedo = S::PL == 2;
     constexpr int kPitch = kSolveBlk + 1, kArea = kSolveBlk * kPitch, kWarps = kFactorThreads / 32;
     // Diagonal block (r, c) at c * kPitch + r, the rows of its factor's inverse (r, c) at r * kPitch + c
-    // before their scaling, both in place; planes kArea apart.  First the warps' transposing tiles.
-    __shared__ float sh[kWarps * kArea];
+    // before their scaling, both in place; planes kArea apart.
+    __shared__ float sh[2 * S::PL * kArea];
     __shared__ float sPiv[256];
     __shared__ int sBad;
-    static_assert(2 * S::PL <= kWarps, "diagonal block and inverse fit the tiles");
     float *sD = sh, *sE = sh + S::PL * kArea;
     const int g = blockIdx.x;
     if (kRedo && flags[g] != kSolveRedo) return;
@@ -198,20 +197,18 @@ __global__ void __launch_bounds__(kFactorThreads, 2) fit_factor_kernel(const flo
     const Blocks<S> L{scratch + (size_t)g * solve_blocks(in) * Blocks<S>::SZ, nb};
     const float* gg = G + (size_t)g * in * in;
     if (threadIdx.x == 0) sBad = 0;
-    // lower blocks of X^T X (only the lower triangle of the sums is kept), transposed tile by tile
+    // lower blocks of X^T X: element (r, c) of the sums is at c * in + r, as in the blocks
     for (int t = warp; t < nb * (nb + 1) / 2; t += kWarps) {
         int i = 0;
         while ((i + 1) * (i + 2) / 2 <= t) ++i;
         const int j = t - i * (i + 1) / 2;
-        float* tile = sh + warp * kArea;
-        __syncwarp();
-#pragma unroll 8
-        for (int r = 0; r < kSolveBlk; ++r)
-            tile[r * kPitch + lane] = gg[(size_t)(i * kSolveBlk + r) * in + j * kSolveBlk + lane];
-        __syncwarp();
+        const float* from = gg + (size_t)j * kSolveBlk * in + i * kSolveBlk + lane;
         float* f = L.F(i, j) + lane;
-#pragma unroll 8
-        for (int c = 0; c < kSolveBlk; ++c) S::make(tile[lane * kPitch + c]).store(f + c * kSolveBlk, kPlane);
+        float x[kSolveBlk];   // all loads before the first store, which might alias them
+#pragma unroll
+        for (int c = 0; c < kSolveBlk; ++c) x[c] = from[(size_t)c * in];
+#pragma unroll
+        for (int c = 0; c < kSolveBlk; ++c) S::make(x[c]).store(f + c * kSolveBlk, kPlane);
     }
     __syncthreads();
 

@@ -336,6 +336,33 @@ def test_blocked_solve_sizes_match_a_double_solve(ds, kl, dt, spread):
             assert _rel(got, ref) <= 16 * (T + 4 * n_in) * 2.0 ** -24, (kv, j, _rel(got, ref))
 
 
+def test_wide_systems_from_tensor_core_sums_match_a_double_solve():
+    """384 unknowns (three source layers of 128 channels): three row blocks of tensor-core sums, solved in
+    double.  bf16 rows without rotation are exact inputs, so only W's rounding to bf16 (2^-9 an element)
+    and the fp32 sums (cond(X)^2 < 16 at T = 4 in, T rounding errors) remain."""
+    import torch
+    kl, ds, dt = 3, 128, 128
+    n_in = kl * ds
+    T = 4 * n_in + 5
+    gen = torch.Generator(device="cuda").manual_seed(9)
+    rnd = lambda d: torch.randn((1, 1, T, d), device="cuda", generator=gen).to(torch.bfloat16)
+    src = [[rnd(ds) for _ in range(2 * kl)] for _ in range(2)]
+    tgt = [[rnd(dt) for _ in range(2)] for _ in range(2)]
+    lmap = [[j * kl + k for k in range(kl)] for j in range(2)]
+    f = kvx.Fitter(synth.ModelGeom(2 * kl, 1, ds, 0.0), synth.ModelGeom(2, 1, dt, 0.0), 0.0, layer_map=lmap,
+                   layers_per_target=kl)
+    i32 = lambda x: torch.tensor(x, dtype=torch.int32, device="cuda")
+    f.accumulate(src[0], src[1], i32([T]), i32([0, T]), T, tgt[0], tgt[1])
+    w = [torch.zeros((2, 1, n_in, dt), dtype=torch.bfloat16, device="cuda") for _ in range(2)]
+    assert f.solve(w[0], w[1]) == 0
+    for kv in range(2):
+        for j in range(2):
+            X = torch.cat([src[kv][l][0, 0] for l in lmap[j]], dim=1).double().cpu().numpy()
+            ref = np.linalg.lstsq(X, tgt[kv][j][0, 0].double().cpu().numpy(), rcond=None)[0]
+            got = w[kv][j, 0].double().cpu().numpy()
+            assert _rel(got, ref) <= 2.0 ** -9 + 16 * T * 2.0 ** -24, (kv, j, _rel(got, ref))
+
+
 def test_fit_two_calls_chunked_and_paged_agree_with_one_call():
     """Sums over calibration calls and accumulation passes add up: one call, two calls, a
     small chunk (several passes) and a paged target cache give the same W (fp32 summation
