@@ -319,14 +319,16 @@ KVX_API int32_t kvx_launches_per_translate(const kvx_translator* tr);
  * the next call only. */
 KVX_API kvx_status kvx_debug_stall_next_translate(kvx_translator* tr, int32_t unit, int32_t wait_us);
 
-/* Diagnostics of the token-span plan of the most recent kvx_translate on this translator, when
- * that call ran the span kernel (its last chunk of up to 65536 target tokens).  The span kernel
+/* Diagnostics of the token-span windows of the most recent kvx_translate on this translator, when
+ * that call ran a span kernel (its last chunk of up to 65536 target tokens).  The window kernel
  * stages the source rows of each 32-token sub-tile as one window of consecutive rows (at most
  * 48); a token whose span lies outside its sub-tile's window (a window cut at the cap, a span
- * in another sequence, a non-monotone span) is gathered from global memory instead.
+ * in another sequence, a non-monotone span) is gathered from global memory instead.  The
+ * row-gather kernel, which takes most geometries, copies rows one by one and has no windows;
+ * its calls leave the same counts, as a description of the spans.
  *   counts: host int64[4] = {sub-tiles, tokens staged in their window, tokens gathered from
  *   global memory, sub-tiles with at least one such token}.
- * Synchronises stream.  KVX_ERR_INVALID_ARG when the last call did not run the span kernel. */
+ * Synchronises stream.  KVX_ERR_INVALID_ARG when the last call did not run a span kernel. */
 KVX_API kvx_status kvx_span_plan_stats(kvx_translator* tr, void* stream, int64_t* counts);
 
 /* ------------------------------------------------------------------------------------------

@@ -44,8 +44,8 @@ void tc_plan_layout(int T_total, int plan_tokens, int* nsub, int* ent_off);
 cudaError_t launch_translate_tc(const TranslateParams& P, const TcConfig& cfg, int num_sms, void* plan,
                                 int plan_tokens, cudaStream_t stream, int* launches);
 
-// spans over gathered source rows (kvx_tc_rows.cu): grouped inputs of up to 256 channels, whole-head
-// rotations.  Same chunks and launches as launch_translate_tc; it also leaves the window plan.
+// spans over gathered source rows (kvx_tc_rows.cu): one head per unit, inputs of up to 256 channels or a
+// multiple of 256, whole-head rotations.  Same chunks and launches as launch_translate_tc; it also leaves the window plan.
 bool rows_supported(int in_dim, int dt, int ds, int share);
 // one head's rows lie within 2^32 16-byte units, as the plan's row offsets count them
 bool rows_offsets_fit(const TranslateParams& P);

@@ -1,4 +1,7 @@
-// kvx_tc.cu -- tensor-core translation kernel for sm_103a (tcgen05 / TMEM / bulk copies).
+// kvx_tc.cu -- tensor-core translation kernel over windows of source rows (tcgen05 / TMEM / bulk copies).
+//
+// It serves what the row-gather kernel (kvx_tc_rows.cu) does not take: units of several heads (the
+// dense form), partial rotary heads, and input widths that are not one or several groups of 256.
 //
 // The per-(target layer, target KV head, K|V) projection of T_theta (paper
 // Section 5) is a dense [T x in] . [in x d_t] contraction; everything around it
