@@ -233,6 +233,10 @@ translate_tc_kernel(const __grid_constant__ TranslateParams P, const __grid_cons
     const int lane = threadIdx.x & 31;
     auto bar = [&](int i) { return smem_u32(&sBar[i]); };
 
+    // The walk, worked out once and copied by every role: its 64-bit divisions in each of them were a fifth of
+    // the kernel's code (dense form, 70B -> 7B shapes, 8192 tokens: 894 us with them, 879 without).
+    Walker* sWalker = reinterpret_cast<Walker*>(smem + L.off_misc + 16);
+    if (threadIdx.x == 32) sWalker->start(L, P.Ht);
     if (threadIdx.x == 0) {
         *sAbort = 0;
         for (int i = 0; i < kMaxB; ++i) {
@@ -314,7 +318,7 @@ translate_tc_kernel(const __grid_constant__ TranslateParams P, const __grid_cons
         uint32_t wphase = 0;       // how often the slots have been cycled, mod 2
         bool ok = true;
         Walker wk;
-        wk.start(L, P.Ht);
+        wk = *sWalker;
         // window headers of the current unit's sub-tiles (lane sq), loaded one unit ahead
         int4 hd = make_int4(0, 0, 0, 0);
         if (wk.more() && lane < kSubPerTile) hd = __ldg(L.plan_hdr + wk.x.tile * kSubPerTile + lane);
@@ -389,7 +393,7 @@ translate_tc_kernel(const __grid_constant__ TranslateParams P, const __grid_cons
             uint32_t b_cnt = 0, pcount = 0, a_cnt = 0;   // B slot b_cnt % n_b, phase (b_cnt / n_b) & 1
             bool ok = true;
             Walker wk;
-            for (wk.start(L, P.Ht); wk.more() && ok; wk.next()) {
+            for (wk = *sWalker; wk.more() && ok; wk.next()) {
                 const Unit& x = wk.x;
                 if (!b_stream && x.g != cur_g) {
                     if (!W.wait(bar(kBarBFull), b_cnt & 1)) break;
@@ -456,7 +460,7 @@ translate_tc_kernel(const __grid_constant__ TranslateParams P, const __grid_cons
             uint32_t b_loads = 0;
             bool ok = true;
             Walker wk;
-            for (wk.start(L, P.Ht); wk.more() && ok; wk.next()) {
+            for (wk = *sWalker; wk.more() && ok; wk.next()) {
                 const Unit& x = wk.x;
                 for (int q = 0; q < L.r_heads && ok; ++q)
                     for (int p = 0; p < NP; ++p) {
@@ -491,7 +495,7 @@ translate_tc_kernel(const __grid_constant__ TranslateParams P, const __grid_cons
         uint32_t pcount = 0;
         bool ok = true;
         Walker wk;
-        for (wk.start(L, P.Ht); wk.more() && ok; wk.next()) {
+        for (wk = *sWalker; wk.more() && ok; wk.next()) {
             const Unit& x = wk.x;
             // resolve the output row while the tile is still being computed
             const int tp = L.t_begin + x.tile * kTileM + m;
@@ -514,6 +518,7 @@ translate_tc_kernel(const __grid_constant__ TranslateParams P, const __grid_cons
                 if (lane == 0) mbar_arrive(bar(kBarPair + quad * 2));
                 if (!W.wait(bar(kBarPair + quad * 2), pcount & 1)) { ok = false; break; }
                 const uint32_t taddr = tmem_base + ((uint32_t)(quad * 32) << 16) + buf * (uint32_t)L.n_tile;
+#pragma unroll 1
                 for (int pc = pc_begin; pc < pc_end; pc += 8) {
                     float2 csn[8];
                     if (rot && pc + 8 < pc_end) rope_cs_vec<8>(sTurnT, pt, nt * hw + pc + 8, csn);
@@ -581,7 +586,7 @@ translate_tc_kernel(const __grid_constant__ TranslateParams P, const __grid_cons
         uint32_t wphase = 0;
         bool ok = true;
         Walker wk;
-        for (wk.start(L, P.Ht); wk.more() && ok; wk.next()) {
+        for (wk = *sWalker; wk.more() && ok; wk.next()) {
             const Unit& x = wk.x;
             const bool rot = x.kv == 0 && P.rs.enabled && lane_rot;
             for (int q = 0; q < L.r_heads && ok; ++q) {
@@ -820,7 +825,7 @@ bool tc_layout(int in_dim, int dt, int ds, int share, TcLaunch& L)
         L.off_stage = take(kTileM * L.stage_row_bytes, 128);
         L.off_meta = take(kNumSlots * kSub * sizeof(int4), 16);
         L.off_bar = take(kNumBars * 8, 8);
-        L.off_misc = take(16, 16);
+        L.off_misc = take(16 + sizeof(Walker), 16);
         L.off_seq = take((2 * kMaxSeqCache + 1) * sizeof(int), 16);
         L.off_turns = take((unsigned)(ds / 2 + dt / 2) * 8, 16);
         L.off_ring = (off + 127) / 128 * 128;
