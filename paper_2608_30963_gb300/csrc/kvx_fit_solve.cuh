@@ -14,8 +14,8 @@
 // Bound: the chain of block columns of one group (the factor) and FMA issue (the solves).  All loops
 // are kept rolled and small: with the diagonal block and the rows below it unrolled in registers,
 // instruction fetch was most of the factor's time.
-// Measured, factor and solves: 112 systems of 256 x 128 in fp32 151 and 149 us (2.0 ms with an unblocked
-// factor and one thread per right-hand side); 208 systems of 128 x 256 in pairs 220 and 502 us, the
+// Measured, factor and solves: 112 systems of 256 x 128 in fp32 151 and 122 us (2.0 ms with an unblocked
+// factor and one thread per right-hand side); 208 systems of 128 x 256 in pairs 220 and 464 us, the
 // latter near the fp32 pipe's rate.
 //
 // Arithmetic is a parameter.  F32: fp32, for systems the pivots show to be well conditioned.  Pair:
@@ -31,7 +31,7 @@ namespace {
 
 constexpr int kSolveBlk = 32;
 constexpr int kFactorThreads = 256;
-constexpr int kTrsmWarps = 8;
+constexpr int kTrsmWarps = 4;   // 32 right-hand sides a CTA: 448 CTAs for 112 groups spread evenly over 152 SMs (122 us; 64 a CTA: 149)
 constexpr int kTrsmStages = 3;  // blocks of L in shared memory
 constexpr int kTrsmCols = 8;    // right-hand sides per warp
 
@@ -473,7 +473,7 @@ __device__ __forceinline__ void copy16(float* dst, const float* src)
 // C: X^T Y, column-major [dt][in]; W out in the cache dtype, [in][dt] per group.  dt is a multiple of the
 // CTA's kTrsmWarps * kTrsmCols columns.
 template <class S, typename T>
-__global__ void __launch_bounds__(kTrsmWarps * 32, 2) fit_trsm_kernel(const float* __restrict__ C,
+__global__ void __launch_bounds__(kTrsmWarps * 32, 4) fit_trsm_kernel(const float* __restrict__ C,
                                                                       const float* __restrict__ scratch, T* wk, T* wv,
                                                                       int in, int dt, const int* __restrict__ flags)
 {
