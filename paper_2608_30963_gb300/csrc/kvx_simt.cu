@@ -5,14 +5,14 @@
 //      head in the dense form, of one or several source layers), undo the source RoPE (K), take
 //      the span mean -> A[tile][in] (fp32, shared memory);
 //   2. projection A . W[j,h] with a register tile of TR tokens x 8 channels a thread; W passes
-//      through shared memory 16 input rows at a time, the next 16 on their way in registers;
+//      through shared memory 8 or 16 input rows at a time, the next ones on their way in registers;
 //   3. the target RoPE (K) and the store, straight from the registers: a thread's 8 channels are 4
 //      rotary pairs.
 // It serves the float32 caches and any geometry the tensor-core kernel does not take.  Paper:
 // Section 5 (T_theta per layer and KV head).
 //
 // Bound: fp32 FMA issue (128 a clock and SM).  Each output is one accumulator in ascending input
-// order.  1000 tokens of 7B -> 1.5B shapes (3.7 G FMA): 211 us; 608 us with a thread per output channel
+// order.  1000 tokens of 7B -> 1.5B shapes (3.7 G FMA): 201 us; 608 us with a thread per output channel
 // and scalar reads of A and W.
 #include "kvx_common.cuh"
 #include "kvx_kernels.h"
@@ -20,13 +20,15 @@
 namespace kvx {
 
 constexpr int kSimtThreads = 128;
-constexpr int kSimtK = 16;          // input rows of W per shared-memory block
 constexpr int kSimtPad = 4;         // floats between two rows of A: 16-byte reads of two rows miss each other's banks
 constexpr int kSimtSmemMax = 200 * 1024;
 
 // Register tile by slots per CTA (rotary pairs: 32 for d_t = 64, else 64): 4 slots (8 channels) a
 // thread, so 8 or 16 threads across the channels and 16 or 8 groups of tokens.
 constexpr int simt_groups(int slots) { return kSimtThreads / (slots / 4); }
+// Input rows of W per shared-memory block: 8 under 32-token tiles, which leaves room for a fifth CTA an SM
+// (201 against 210 us for the case above), 16 under 16-token tiles, whose chain of blocks counts.
+__host__ __device__ constexpr int simt_k(int tm) { return tm == 32 ? 8 : 16; }
 
 // 4 consecutive elements; VEC: 16-byte aligned rows, else element by element.
 template <bool VEC>
@@ -62,7 +64,7 @@ __device__ __forceinline__ void store4(__nv_bfloat16* p, float4 x)
     }
 }
 // (c0, c1) += x (w0, w1): one packed instruction for two fp32 FMAs, each rounded as fmaf.  The packed
-// form halves the issue slots of the projection (236 to 211 us for the case above).
+// form halves the issue slots of the projection (236 to 211 us for the case above, four CTAs an SM).
 __device__ __forceinline__ void fma2(float& c0, float& c1, float x, float w0, float w1)
 {
     asm("{\n\t.reg .b64 a, b, c;\n\tmov.b64 a, {%2, %2};\n\tmov.b64 b, {%3, %4};\n\tmov.b64 c, {%0, %1};\n\t"
@@ -88,7 +90,7 @@ __device__ __forceinline__ void rotate(float& lo, float& hi, float2 cs)
 template <typename T, int SLOTS, int TR, bool VEC>
 __global__ void __launch_bounds__(kSimtThreads) translate_simt_kernel(const __grid_constant__ TranslateParams P)
 {
-    constexpr int CG = SLOTS / 4, RG = kSimtThreads / CG, TM = RG * TR;
+    constexpr int CG = SLOTS / 4, RG = kSimtThreads / CG, TM = RG * TR, kSimtK = simt_k(TM);
     constexpr int WROW = 2 * SLOTS;                              // floats of one staged row of W
     constexpr int WPT = kSimtK * WROW / 4 / kSimtThreads;        // float4 of a staged block per thread
     extern __shared__ float smem[];
@@ -282,7 +284,7 @@ cudaError_t launch_fold_low_rank(const void* a, const void* b, void* w, int n, i
 namespace {
 size_t simt_smem(int in_dim, int slots, int tm)
 {
-    return ((size_t)tm * (in_dim + kSimtPad) + 2 * (size_t)kSimtK * 2 * slots) * sizeof(float);
+    return ((size_t)tm * (in_dim + kSimtPad) + 2 * (size_t)simt_k(tm) * 2 * slots) * sizeof(float);
 }
 int simt_slots(int dt) { return dt == 64 ? 32 : 64; }
 
@@ -322,7 +324,7 @@ size_t simt_smem_bytes(int in_dim, int dt)
 cudaError_t launch_translate_simt(const TranslateParams& P, int dtype, cudaStream_t stream)
 {
     // 32-token tiles where they give two CTAs an SM (152 SMs) and A fits shared memory, else 16: four CTAs of
-    // 32 tokens an SM overlap their phases (211 us; two of 64 tokens and 128 threads 256, of 256 threads 227),
+    // 32 tokens an SM overlap their phases (211 us, with 8 rows of W a block five and 199; two of 64 tokens and 128 threads 256, of 256 threads 227),
     // and below two CTAs an SM the chain of one CTA counts
     const long long tiles = (long long)((P.T_total + 31) / 32) * P.Ht * (P.dt / (2 * simt_slots(P.dt))) * P.Lt * 2;
     const bool big = tiles >= 2 * 152 && simt_smem(P.in_dim, simt_slots(P.dt), 32) <= (size_t)kSimtSmemMax;
