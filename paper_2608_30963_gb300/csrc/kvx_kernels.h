@@ -25,7 +25,6 @@ struct TcConfig {
     int threads;
     int ok;            // geometry supported
     int hpu;           // target heads of one unit of the window kernel
-    int streamed;      // its weights stream in pieces (else one resident image per group)
 };
 // share: target heads that read the same input rows (share_heads); it decides how many heads
 // one unit of the span kernel covers and so the weight images' output split n_tile.

@@ -847,13 +847,12 @@ bool tc_layout(int in_dim, int dt, int ds, int share, TcLaunch& L)
 TcConfig tc_config(int in_dim, int dt, int ds, int share)
 {
     TcLaunch L{};
-    TcConfig c{0, 0, 0, kThreads, 0, 1, 0};
+    TcConfig c{0, 0, 0, kThreads, 0, 1};
     if (!tc_layout(in_dim, dt, ds, share, L)) return c;
     c.n_tile = L.n_tile;
     c.n_split = L.n_split;
     c.smem_bytes = kSmemMax;
     c.hpu = L.hpu;
-    c.streamed = L.n_b > 1;
     c.ok = 1;
     return c;
 }

@@ -88,7 +88,7 @@ struct TilePlan {
 struct RowsLaunch {
     int n_tile, n_split, nslots, share;
     int nblk, kgs;         // K-blocks of a K group (at most 256 channels), K groups of an input row
-    int nb;                // weight ring slots, each a K-block; 0: the image stays resident
+    int nb;                // weight ring slots, each a K-block (several K groups); 0: the image stays resident
     int m_tiles;
     int side_rows;         // further rows the side buffer holds
     const TilePlan* tiles; // [tile]
@@ -800,10 +800,11 @@ bool rows_layout(int in_dim, int dt, int ds, int share, RowsLaunch& L)
     L.nblk = width / kBlockK;
     L.kgs = in_dim / width;
     L.b_bytes = (unsigned)(in_dim * L.n_tile * 2);
-    // weights: the group's image where it fits, else a ring of K-blocks
+    // weights: the group's image with one K group, else a ring of K-blocks (also where the image of several K
+    // groups would fit: 512 channels onto 64), since only the streaming form walks K groups
     constexpr unsigned kWeightBytes = 65536;
     L.nb = 0;
-    if (c.streamed) {
+    if (L.kgs > 1) {
         L.nb = (int)(kWeightBytes / (unsigned)(L.n_tile * 128));
         if (L.nb > kMaxB) L.nb = kMaxB;
     }
@@ -848,7 +849,7 @@ cudaError_t launch_rows_v(int grid, cudaStream_t stream, const TranslateParams& 
 template <int HS, int HEADS>
 cudaError_t launch_rows(int grid, cudaStream_t stream, const TranslateParams& P, const RowsLaunch& L)
 {
-    return L.nb ? launch_rows_v<HS, HEADS, true>(grid, stream, P, L) : launch_rows_v<HS, HEADS, false>(grid, stream, P, L);
+    return L.kgs > 1 ? launch_rows_v<HS, HEADS, true>(grid, stream, P, L) : launch_rows_v<HS, HEADS, false>(grid, stream, P, L);
 }
 
 }  // namespace

@@ -587,3 +587,38 @@ def test_gathered_rows_kernel_edges(Hs, ds, Ht, dt, law, T):
     assert a[:, :, 1].abs().max() == 0 and b[:, :, 1].abs().max() == 0   # no source tokens: zero rows
     for kv in range(2):
         assert (a[kv] - b[kv]).norm() <= 2.0 ** -8 * 1.5 * b[kv].norm(), (kv, (a[kv] - b[kv]).norm() / b[kv].norm())
+
+
+@pytest.mark.parametrize("spans", [False, True])
+@pytest.mark.parametrize("Hs,ds,Ht,dt,kl", [(8, 64, 1, 64, 1), (4, 128, 1, 64, 1), (2, 256, 1, 64, 1), (4, 128, 2, 64, 2),
+                                            (1, 128, 1, 64, 4), (8, 128, 2, 64, 2), (8, 128, 1, 64, 1), (4, 128, 1, 256, 1)])
+def test_inputs_of_several_k_groups_reach_every_channel(Hs, ds, Ht, dt, kl, spans):
+    """Inputs of 512 and 1024 channels (one, two and four source layers), with spans and one tokenizer.  512
+    onto 64-channel heads has a weight image that would fit shared memory whole, and still takes two K groups.
+    Against the CUDA-core kernel: both sum in fp32, the tensor-core kernels round their input rows to bf16
+    first, a relative 2^-9 each."""
+    L, T = 3, 300
+    rng = np.random.default_rng(23)
+    n = rng.integers(1, 4, size=T) if spans else np.ones(T, int)
+    hi = np.cumsum(n)
+    S = int(hi[-1])
+    i32 = lambda x: torch.tensor(np.asarray(x), dtype=torch.int32, device="cuda")
+    gen = torch.Generator(device="cuda").manual_seed(4)
+    rnd = lambda *sh: torch.randn(sh, device="cuda", generator=gen).to(torch.bfloat16)
+    n_in = kl * max(1, Hs // Ht) * ds
+    src = [[rnd(1, Hs, S, ds) for _ in range(L * kl)] for _ in range(2)]
+    w = [rnd(L, Ht, n_in, dt) for _ in range(2)]
+    sp = dict(span_lo=i32(hi - n), span_hi=i32(hi)) if spans else {}
+    outs = []
+    for path in (kvx.KVX_PATH_TCGEN05, kvx.KVX_PATH_SIMT):
+        tr = kvx.Translator(synth.ModelGeom(L * kl, Hs, ds, 1e4), synth.ModelGeom(L, Ht, dt, 1e6), w[0], w[1],
+                            layer_map=[[j * kl + k for k in range(kl)] for j in range(L)], path=path, layers_per_target=kl)
+        dst = [[torch.full((1, Ht, T, dt), float("nan"), dtype=torch.bfloat16, device="cuda") for _ in range(L)] for _ in range(2)]
+        tr.translate(src[0], src[1], i32([S]), i32([0, T]), T, dst[0], dst[1], **sp)
+        torch.cuda.synchronize()
+        assert tr.device_status() == 0
+        outs.append(torch.stack([torch.stack(d) for d in dst]).double())
+    a, b = outs
+    assert not a.isnan().any() and not b.isnan().any()
+    for kv in range(2):
+        assert (a[kv] - b[kv]).norm() <= 2.0 ** -8 * 1.5 * b[kv].norm(), (kv, (a[kv] - b[kv]).norm() / b[kv].norm())
