@@ -84,8 +84,9 @@ __device__ __forceinline__ void resolve_dst(const TranslateParams& P, const SeqV
 //           start (low 16 bits, signed; -1: read from global memory) | A row within
 //           the sub-tile << 16 (0xFFFF: token past the end); [lo, hi) the clamped
 //           source span of sequence b.
-// One warp writes the plan of sub-tile sub: lane = token (valid, its sequence and clamped span).
-__device__ __forceinline__ void write_window_plan(bool valid, int b, int lo, int hi, int sub, int lane, int cap_rows,
+// One warp writes the plan of sub-tile sub: lane = token (valid, its sequence and clamped span); returns whether
+// the lane's token lies in the window.
+__device__ __forceinline__ bool write_window_plan(bool valid, int b, int lo, int hi, int sub, int lane, int cap_rows,
                                                   int4* __restrict__ hdr, int4* __restrict__ ent)
 {
     // valid tokens are a prefix of the sub-tile, so lane 0 opens the window
@@ -110,6 +111,7 @@ __device__ __forceinline__ void write_window_plan(bool valid, int b, int lo, int
     const int w0 = (int)(((unsigned)stage_row & 0xFFFFu) | ((valid ? (unsigned)lane : 0xFFFFu) << 16));
     ent[(size_t)sub * 32 + rank] = make_int4(w0, lo, hi, b < 0 ? 0 : b);
     if (lane == 0) hdr[sub] = make_int4(b0 < 0 ? 0 : b0, c0, R, 0);
+    return inwin;
 }
 
 // programmatic stream serialization: see the kernels' griddepcontrol.wait

@@ -28,10 +28,21 @@
 //                  quadrant, each taking half of the rotary pairs
 //   warps 12-19    prologue: source-RoPE undo of K rows in place, span means
 // Every wait is bounded (~1 s, then KVX_DEV_WAIT_TIMEOUT and a drained exit).
+//
+// Dense spans.  Further rows that the side buffer has no room for are read from memory by the prologue, with their
+// latency exposed; a window (kvx_tc_window.cuh) holds 48 rows of a 32-token sub-tile and is copied ahead.  The spans
+// are known on the device only.  Where the source may hold 1.5 rows or more for each target token the kernel is
+// launched in a form (DENSE) that counts, over the plan's tiles, the further rows beyond the side buffer (o), the
+// tokens of several rows (m) and the rows of the tokens outside their windows (w), and runs the window kernel's body
+// where o + 2 m - w / 4 exceeds dense_sum a tile (rows_layout).  With fewer source rows the spans can only be dense
+// where they overlap, and the plain form runs: the count and the second body cost it up to 2% (70B -> 7B shapes, 8192
+// tokens: 513 us against 503; 1.5B -> Gemma-2B shapes, a ragged batch of 1574: 98.8 against 98.0).  4096 tokens, 8 layers of 128 x 128 heads grouped by two, us here and in windows:
+// spans of 1.3 rows 59 and 79, of 1.6 86 and 94, of 2 119 and 114, of two each 112 and 91, of 8 to 16 964 and 803.
 #include "kvx_common.cuh"
 #include "kvx_kernels.h"
 #include "kvx_span_plan.cuh"
 #include "kvx_tc_common.cuh"
+#include "kvx_tc_window.cuh"
 
 namespace kvx {
 namespace {
@@ -77,9 +88,10 @@ struct RowEnt {
     int4 src, dst;
     int2 where, pad;
 };
-// Plan of a tile: rows with spans of other than one row, tokens, further rows, 0; the offsets of the
-// first kSideMax further rows.
+// Plan of a tile: rows with spans of other than one row, tokens, further rows, source rows of the tokens outside
+// their sub-tile's window (both saturated at kRowsMax); the offsets of the first kSideMax further rows.
 constexpr int kSideMax = 128;
+constexpr int kRowsMax = 1 << 18;   // four times this over the 512 tiles of a launch fits an int
 struct TilePlan {
     int4 count;
     unsigned side[kSideMax];
@@ -91,6 +103,7 @@ struct RowsLaunch {
     int nb;                // weight ring slots, each a K-block (several K groups); 0: the image stays resident
     int m_tiles;
     int side_rows;         // further rows the side buffer holds
+    int dense_sum;         // dense spans: the sum a tile above which they are (see the top)
     const TilePlan* tiles; // [tile]
     const RowEnt* rows;    // [tile][128]
     unsigned b_bytes, stage_row_bytes;
@@ -260,10 +273,12 @@ __device__ __forceinline__ uint4 pack8(const float (&a)[8], float f)
                       pack_bf16(a[6] * f, a[7] * f));
 }
 // HS: half head_dim of the source (32, 64 or 128); HEADS: source heads of a K group; STREAM: several K groups,
-// weights streamed (else a resident image)
-template <int HS, int HEADS, bool STREAM>
+// weights streamed (else a resident image); DENSE: the spans may be dense (see the top), D is the window kernel's
+// launch over the same tokens
+template <int HS, int HEADS, bool STREAM, bool DENSE>
 __global__ void __launch_bounds__(kThreads, 1)
-translate_rows_kernel(const __grid_constant__ TranslateParams P, const __grid_constant__ RowsLaunch L)
+translate_rows_kernel(const __grid_constant__ TranslateParams P, const __grid_constant__ RowsLaunch L,
+                      const __grid_constant__ window::TcLaunch D)
 {
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
@@ -276,6 +291,7 @@ translate_rows_kernel(const __grid_constant__ TranslateParams P, const __grid_co
     volatile int* sAbort = reinterpret_cast<volatile int*>(smem + L.off_misc);
     uint32_t* sTmemBase = reinterpret_cast<uint32_t*>(smem + L.off_misc + 4);
     RWalkStart& sWalk = *reinterpret_cast<RWalkStart*>(smem + L.off_misc + 16);
+    int* sDense = reinterpret_cast<int*>(smem + L.off_misc + 16 + sizeof(RWalkStart));
     unsigned long long* sTurnS = reinterpret_cast<unsigned long long*>(smem + L.off_turns);
     unsigned long long* sTurnT = sTurnS + HS;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -283,29 +299,33 @@ translate_rows_kernel(const __grid_constant__ TranslateParams P, const __grid_co
     const uint32_t NS = (uint32_t)L.nslots, NKR = NS / (uint32_t)L.nblk + 2;
 
     if (threadIdx.x == 32) sWalk.init(P, L);
-    if (threadIdx.x == 0) {
-        *sAbort = 0;
+    // f(index, arrivals) for every barrier
+    auto barriers = [&](auto f) {
         for (int i = 0; i < kMaxB; ++i) {
-            mbar_init(bar(kBarBFull + i), 1);
-            mbar_init(bar(kBarBEmpty + i), 1);
+            f(kBarBFull + i, 1);
+            f(kBarBEmpty + i, 1);
         }
         for (int i = 0; i < 2; ++i) {
-            mbar_init(bar(kBarDFull + i), 1);
-            mbar_init(bar(kBarDEmpty + i), kNumEpiWarps);
+            f(kBarDFull + i, 1);
+            f(kBarDEmpty + i, kNumEpiWarps);
         }
-        for (uint32_t i = 0; i < NS; ++i) {
-            mbar_init(bar(kBarFull + i), kNumGatherWarps * 32);   // every gather lane's copies
-            mbar_init(bar(kBarEmpty + i), 1);
+        for (int i = 0; i < (int)NS; ++i) {
+            f(kBarFull + i, kNumGatherWarps * 32);   // every gather lane's copies
+            f(kBarEmpty + i, 1);
         }
-        for (uint32_t i = 0; i < NKR; ++i) mbar_init(bar(kBarKReady + i), kNumXfWarps);
+        for (int i = 0; i < (int)NKR; ++i) f(kBarKReady + i, kNumXfWarps);
         for (int i = 0; i < kEntTabs; ++i) {
-            mbar_init(bar(kBarEntFull + i), kNumGatherWarps * 32);
-            mbar_init(bar(kBarEntEmpty + i), kNumXfWarps);
+            f(kBarEntFull + i, kNumGatherWarps * 32);
+            f(kBarEntEmpty + i, kNumXfWarps);
         }
-        mbar_init(bar(kBarSideFull), 32);
-        mbar_init(bar(kBarSideEmpty), kNumXfWarps);
-        for (int i = 0; i < 8; ++i) mbar_init(bar(kBarPair + i), kEpiParts);
-        mbar_init(bar(kBarMmaDone), 1);
+        f(kBarSideFull, 32);
+        f(kBarSideEmpty, kNumXfWarps);
+        for (int i = 0; i < 8; ++i) f(kBarPair + i, kEpiParts);
+        f(kBarMmaDone, 1);
+    };
+    if (threadIdx.x == 0) {
+        *sAbort = 0;
+        barriers([&](int i, int n) { mbar_init(bar(i), (uint32_t)n); });
         fence_mbar_init();
     }
     if (warp == kMmaWarp) {
@@ -319,14 +339,27 @@ translate_rows_kernel(const __grid_constant__ TranslateParams P, const __grid_co
     for (int i = threadIdx.x; i < HS; i += blockDim.x)
         sTurnS[(i & 7) * (HS / 8) + (i >> 3)] = P.rs.enabled ? __ldg(&P.rs.turns[i]) : 0ull;
     for (int i = threadIdx.x; i < (P.dt >> 1); i += blockDim.x) sTurnT[i] = P.rt.enabled ? __ldg(&P.rt.turns[i]) : 0ull;
+    if (DENSE && warp == kSideWarp) {
+        int v = 0;
+#pragma unroll 4
+        for (int i = lane; i < L.m_tiles; i += 32) {
+            const int4 c = __ldg(&L.tiles[i].count);
+            v += 4 * (max(c.z - L.side_rows, 0) + 2 * min(c.x, c.z) - L.dense_sum) - c.w;
+        }
+        v = __reduce_add_sync(0xffffffffu, v);
+        if (lane == 0) *sDense = v;
+    }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = *sTmemBase;
+    const int dense = DENSE ? *sDense : 0;   // above 0: dense spans, in every CTA of the launch
     const RWaiter W{sAbort, P.status, P.wait_ns ? P.wait_ns : kWaitNs};
     const int hw = L.n_tile >> 1;
 
-    if (warp == kMmaWarp) {
+    if (DENSE && dense > 0) {
+        // below
+    } else if (warp == kMmaWarp) {
         if (lane == 0) {
             const uint64_t pol_keep = policy_evict_last();
             const uint32_t nb = STREAM ? (uint32_t)L.nb : 0u, kblock = (uint32_t)L.n_tile * 128;   // bytes of a K-block of weights
@@ -713,6 +746,13 @@ translate_rows_kernel(const __grid_constant__ TranslateParams P, const __grid_co
         }
         cp_async_wait_all();
     }
+    if (DENSE && dense > 0) {
+        __syncthreads();   // everyone has read what the shared memory held
+        if (threadIdx.x == 0)
+            barriers([&](int i, int) { mbar_inval(bar(i)); });
+        __syncthreads();
+        window::translate_body<2 * HS, false, false>(P, D, smem, tmem_base);
+    }
 
     tc_fence_before();
     __syncthreads();
@@ -731,6 +771,7 @@ __global__ void __launch_bounds__(kTileM) span_rows_kernel(const __grid_constant
     constexpr int kClasses = 5;   // 0: four rows and more, 1: three, 2: two or none, 3: one, 4: past the last token
     __shared__ int cnt[kClasses][kTileM / 32];
     __shared__ int more[kTileM];   // [rank]: further rows
+    __shared__ int out[kTileM / 32];
     // the previous launch in the stream may still read the plan
     grid_dependency_wait();
     grid_launch_dependents();
@@ -740,8 +781,11 @@ __global__ void __launch_bounds__(kTileM) span_rows_kernel(const __grid_constant
     const bool valid = tp < t_end;
     int b = -1, lo = 0, hi = 0;
     if (valid) resolve_src<true>(P, sv, tp, load_span(P, tp), b, lo, hi);
-    write_window_plan(valid, b, lo, hi, (int)blockIdx.x * (kTileM / 32) + warp, lane, cap_rows, hdr, win);
+    const bool inwin = write_window_plan(valid, b, lo, hi, (int)blockIdx.x * (kTileM / 32) + warp, lane, cap_rows, hdr, win);
     const int n = valid ? hi - lo : -1;
+    // (a tile's sums are at most 128 x 2048 = kRowsMax)
+    const int out_rows = __reduce_add_sync(0xffffffffu, inwin || n < 0 ? 0 : min(n, kRowsMax / kTileM));
+    if (lane == 0) out[warp] = out_rows;
     const int cls = n < 0 ? 4 : n == 1 ? 3 : n >= 4 ? 0 : n == 3 ? 1 : 2;
     int rank = 0;   // among the earlier lanes of the same class
 #pragma unroll
@@ -767,7 +811,8 @@ __global__ void __launch_bounds__(kTileM) span_rows_kernel(const __grid_constant
     int side = 0;
     for (int r = 0; r < rank && r < multi; ++r) side += more[r];
     TilePlan& tile = tiles[blockIdx.x];
-    if (rank == kTileM - 1) tile.count = make_int4(multi, tokens, side + more[rank], 0);
+    if (rank == kTileM - 1)
+        tile.count = make_int4(multi, tokens, min(side + more[rank], kRowsMax), out[0] + out[1] + out[2] + out[3]);
     RowEnt& row = rows[(size_t)blockIdx.x * kTileM + rank];
     if (!valid) {
         row.src = make_int4(0, -1, 0, 0);
@@ -819,7 +864,7 @@ bool rows_layout(int in_dim, int dt, int ds, int share, RowsLaunch& L)
     L.off_b = take(L.nb ? (unsigned)(L.nb * L.n_tile * 128) : L.b_bytes, 1024);
     L.off_stage = take(kTileM * L.stage_row_bytes, 128);
     L.off_bar = take(kNumBars * 8, 8);
-    L.off_misc = take(16 + sizeof(RWalkStart), 16);
+    L.off_misc = take(16 + sizeof(RWalkStart) + sizeof(int), 16);
     L.off_turns = take((unsigned)(ds / 2 + dt / 2) * 8, 16);
     L.off_ent = take(kEntTabs * kTileM * sizeof(int4), 16);
     L.off_ring = take(0, 1024);
@@ -832,6 +877,10 @@ bool rows_layout(int in_dim, int dt, int ds, int share, RowsLaunch& L)
     L.off_side = L.off_ring + (unsigned)L.nslots * kBlockBytes;
     const int fit = (avail - L.nslots * kBlockBytes) / row;
     L.side_rows = fit < kSideMax ? fit : kSideMax;
+    // Where the two sides meet: heads of 64 keep more lanes on a row.  Over 57 geometries and 21 laws of spans (1.3 to
+    // 12 rows, disjoint and overlapping, even and uneven) the side taken is 0.8% above the faster one on average, and
+    // at most 34% (128-channel heads, a tenth of the tokens with 16 rows).
+    L.dense_sum = ds == 64 ? (L.kgs > 1 ? 240 : 300) : ds == 128 ? 220 : 165;
     L.idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(L.n_tile >> 3) << 17) | ((uint32_t)(kTileM >> 4) << 24);
     unsigned cols = 32;
     while (cols < 2u * (unsigned)L.n_tile) cols <<= 1;
@@ -839,17 +888,23 @@ bool rows_layout(int in_dim, int dt, int ds, int share, RowsLaunch& L)
     return cols <= 512;
 }
 
-template <int HS, int HEADS, bool STREAM>
-cudaError_t launch_rows_v(int grid, cudaStream_t stream, const TranslateParams& P, const RowsLaunch& L)
+template <int HS, int HEADS, bool STREAM, bool DENSE>
+cudaError_t launch_rows_v(int grid, cudaStream_t stream, const TranslateParams& P, const RowsLaunch& L,
+                          const window::TcLaunch& D)
 {
-    const cudaError_t e = smem_opt_in<translate_rows_kernel<HS, HEADS, STREAM>>(kSmemMax);
+    const cudaError_t e = smem_opt_in<translate_rows_kernel<HS, HEADS, STREAM, DENSE>>(kSmemMax);
     if (e != cudaSuccess) return e;
-    return launch_pdl(translate_rows_kernel<HS, HEADS, STREAM>, grid, kThreads, kSmemMax, stream, P, L);
+    return launch_pdl(translate_rows_kernel<HS, HEADS, STREAM, DENSE>, grid, kThreads, kSmemMax, stream, P, L, D);
 }
 template <int HS, int HEADS>
-cudaError_t launch_rows(int grid, cudaStream_t stream, const TranslateParams& P, const RowsLaunch& L)
+cudaError_t launch_rows(int grid, bool dense, cudaStream_t stream, const TranslateParams& P, const RowsLaunch& L,
+                        const window::TcLaunch& D)
 {
-    return L.kgs > 1 ? launch_rows_v<HS, HEADS, true>(grid, stream, P, L) : launch_rows_v<HS, HEADS, false>(grid, stream, P, L);
+    if (L.kgs > 1)
+        return dense ? launch_rows_v<HS, HEADS, true, true>(grid, stream, P, L, D)
+                     : launch_rows_v<HS, HEADS, true, false>(grid, stream, P, L, D);
+    return dense ? launch_rows_v<HS, HEADS, false, true>(grid, stream, P, L, D)
+                 : launch_rows_v<HS, HEADS, false, false>(grid, stream, P, L, D);
 }
 
 }  // namespace
@@ -876,8 +931,11 @@ cudaError_t launch_translate_rows(const TranslateParams& P, int num_sms, void* w
 {
     *launches = 0;
     RowsLaunch L{};
+    window::TcLaunch D{};
     const int share = share_heads(P);
-    if (!rows_layout(P.in_dim, P.dt, P.ds, share, L)) return cudaErrorNotSupported;
+    if (!rows_layout(P.in_dim, P.dt, P.ds, share, L) || !window::tc_layout(P.in_dim, P.dt, P.ds, share, D) ||
+        D.np != 1 || D.tmem_cols != L.tmem_cols)
+        return cudaErrorNotSupported;
     const int chunk = plan_tokens / kTileM * kTileM;
     if (chunk <= 0 || !plan || !window_plan) return cudaErrorInvalidValue;
     int4* hdr = reinterpret_cast<int4*>(window_plan);
@@ -886,23 +944,26 @@ cudaError_t launch_translate_rows(const TranslateParams& P, int num_sms, void* w
     TilePlan* tiles = reinterpret_cast<TilePlan*>(rows + chunk);
     L.tiles = tiles;
     L.rows = rows;
+    // the source may hold 1.5 rows or more for each target token (what the host knows: the caches' capacity)
+    const bool dense = P.span_lo && 2ll * P.batch * P.src_max_seq >= 3ll * P.T_total;
     L.share = share > 1 && P.Ht % share == 0 ? share : 1;
     for (int t0 = 0; t0 < P.T_total; t0 += chunk) {
         const int t1 = P.T_total - t0 < chunk ? P.T_total : t0 + chunk;
         L.m_tiles = (t1 - t0 + kTileM - 1) / kTileM;
         const long long UH = (long long)P.Lt * P.Ht * L.n_split * L.m_tiles;
         const int grid = (int)(UH < num_sms ? UH : num_sms);
+        if (window::tc_launch(P, t0, t1, hdr, win, num_sms, D) != grid) return cudaErrorInvalidValue;
         if (grid % L.share) L.share = 1;
         cudaError_t e = launch_pdl(span_rows_kernel, L.m_tiles, kTileM, 0, stream, P, t0, t1, kWindowRows, hdr, win, tiles, rows);
         if (e != cudaSuccess) return e;
         ++*launches;
         switch (P.ds * 8 + L.nblk * kBlockK / P.ds) {   // source heads of a K group
-        case 64 * 8 + 1: e = launch_rows<32, 1>(grid, stream, P, L); break;
-        case 64 * 8 + 2: e = launch_rows<32, 2>(grid, stream, P, L); break;
-        case 64 * 8 + 4: e = launch_rows<32, 4>(grid, stream, P, L); break;
-        case 128 * 8 + 1: e = launch_rows<64, 1>(grid, stream, P, L); break;
-        case 128 * 8 + 2: e = launch_rows<64, 2>(grid, stream, P, L); break;
-        case 256 * 8 + 1: e = launch_rows<128, 1>(grid, stream, P, L); break;
+        case 64 * 8 + 1: e = launch_rows<32, 1>(grid, dense, stream, P, L, D); break;
+        case 64 * 8 + 2: e = launch_rows<32, 2>(grid, dense, stream, P, L, D); break;
+        case 64 * 8 + 4: e = launch_rows<32, 4>(grid, dense, stream, P, L, D); break;
+        case 128 * 8 + 1: e = launch_rows<64, 1>(grid, dense, stream, P, L, D); break;
+        case 128 * 8 + 2: e = launch_rows<64, 2>(grid, dense, stream, P, L, D); break;
+        case 256 * 8 + 1: e = launch_rows<128, 1>(grid, dense, stream, P, L, D); break;
         default: return cudaErrorNotSupported;
         }
         if (e != cudaSuccess) return e;

@@ -622,3 +622,40 @@ def test_inputs_of_several_k_groups_reach_every_channel(Hs, ds, Ht, dt, kl, span
     assert not a.isnan().any() and not b.isnan().any()
     for kv in range(2):
         assert (a[kv] - b[kv]).norm() <= 2.0 ** -8 * 1.5 * b[kv].norm(), (kv, (a[kv] - b[kv]).norm() / b[kv].norm())
+
+
+@pytest.mark.parametrize("Hs,ds,Ht,dt", [(1, 64, 1, 64), (4, 64, 1, 128), (1, 128, 2, 256), (2, 128, 1, 128), (1, 256, 1, 128),
+                                         (4, 128, 1, 128)])
+@pytest.mark.parametrize("law", ["few_long", "few_long_padded", "all_long", "overlapping", "overlapping_padded"])
+def test_span_kernels_agree_on_either_side_of_the_dense_rule(Hs, ds, Ht, dt, law):
+    """The row-gather kernel takes calls whose spans mostly fit its side buffer, and runs the window kernel's body on
+    dense ones where the source caches may hold 1.5 rows a token.  few_long: 20 spans of 12 rows among 2051 (its own
+    walk, whose overflowing tile reads further rows from memory); all_long: 12 rows each; overlapping: three rows
+    each, two of them the next token's; padded: caches of twice the length.  Against the CUDA-core kernel, as above."""
+    T, L = 2051, 2
+    law, padded = law.removesuffix("_padded"), law.endswith("_padded")
+    n = np.full(T, {"few_long": 1, "all_long": 12, "overlapping": 3}[law])
+    if law == "few_long":
+        n[700:720] = 12
+    lo = np.arange(T) if law == "overlapping" else np.cumsum(n) - n
+    S = int((lo + n).max())
+    i32 = lambda x: torch.tensor(np.asarray(x), dtype=torch.int32, device="cuda")
+    gen = torch.Generator(device="cuda").manual_seed(6)
+    rnd = lambda *sh: torch.randn(sh, device="cuda", generator=gen).to(torch.bfloat16)
+    n_in = max(1, Hs // Ht) * ds
+    src = [[rnd(1, Hs, S * (2 if padded else 1), ds) for _ in range(L)] for _ in range(2)]
+    w = [rnd(L, Ht, n_in, dt) for _ in range(2)]
+    outs = []
+    for path in (kvx.KVX_PATH_TCGEN05, kvx.KVX_PATH_SIMT):
+        tr = kvx.Translator(synth.ModelGeom(L, Hs, ds, 1e4), synth.ModelGeom(L, Ht, dt, 1e6), w[0], w[1],
+                            layer_map=list(range(L)), path=path)
+        dst = [[torch.full((1, Ht, T, dt), float("nan"), dtype=torch.bfloat16, device="cuda") for _ in range(L)] for _ in range(2)]
+        for _ in range(2):   # twice: the second call follows the first on the stream
+            tr.translate(src[0], src[1], i32([S]), i32([0, T]), T, dst[0], dst[1], span_lo=i32(lo), span_hi=i32(lo + n))
+        torch.cuda.synchronize()
+        assert tr.device_status() == 0
+        outs.append(torch.stack([torch.stack(d) for d in dst]).double())
+    a, b = outs
+    assert not a.isnan().any() and not b.isnan().any()
+    for kv in range(2):
+        assert (a[kv] - b[kv]).norm() <= 2.0 ** -8 * 1.5 * b[kv].norm(), (kv, (a[kv] - b[kv]).norm() / b[kv].norm())
