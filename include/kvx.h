@@ -347,7 +347,7 @@ KVX_API kvx_status kvx_span_plan_stats(kvx_translator* tr, void* stream, int64_t
  * tensor cores for bf16 caches with in + out <= 512 and in a multiple of 128, X and Y built on
  * chip; on the CUDA cores otherwise), then solves all systems at once (Cholesky factorisation on
  * the device: in fp32 for in <= 256, where a system whose factor shows a condition number above
- * 1e3 is solved again in pairs of floats, about 48 bits; in double above).  Forms as for
+ * 1e3 is solved again in pairs of floats, about 48 bits, or in double; in double above).  Forms as for
  * kvx_translator_create; latent adapters are not fitted (fit W, then factor it if wanted). */
 typedef struct kvx_fitter kvx_fitter;
 
@@ -374,7 +374,7 @@ KVX_API kvx_status kvx_fit_accumulate(kvx_fitter* f, const kvx_src_kv* src, cons
  * the fitter's status word: KVX_DEV_* bits from the accumulation passes (rows left out), 0x20
  * when a system was not positive definite (lambda = 0 with too few tokens; its W is zero), in
  * which case the call returns KVX_ERR_DEVICE_STATUS, and 0x40 (informational) when
- * ill-conditioned systems were solved in pairs of floats.  Calls on one fitter must be ordered
+ * ill-conditioned systems were solved again in more than fp32.  Calls on one fitter must be ordered
  * (one stream, or synchronised by the caller). */
 KVX_API kvx_status kvx_fit_solve(kvx_fitter* f, void* w_k, void* w_v, uint32_t* status_bits, void* stream);
 

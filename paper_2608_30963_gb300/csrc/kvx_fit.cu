@@ -15,9 +15,10 @@
 //   fit_rows_kernel builds X and Y for one pass of up to chunk tokens, then fit_gram_simt_kernel
 //   adds their products into the sums on the CUDA cores.
 // Solve (kvx_fit_solve), in <= 256: a blocked Cholesky factor X^T X + lambda I = L L^T and the two
-//   triangular solves (kvx_fit_solve.cuh) in fp32, and again in pairs of floats (about 48 bits) for
-//   the systems whose factor shows a condition number above 10^3.  Wider systems: fit_solve_kernel,
-//   one CTA per group, in double in global memory.
+//   triangular solves (kvx_fit_solve.cuh) in fp32, again in pairs of floats (about 48 bits) for the
+//   systems whose factor shows a condition number above 10^3, and again in double for those that show
+//   one above 4096 with the channels scaled alike.  Wider systems, and these: fit_solve_kernel, one CTA
+//   per group, in double in global memory.
 #include <math.h>
 #include <stdarg.h>
 #include <stdio.h>
@@ -35,12 +36,15 @@ constexpr int kFitTile = 32;
 constexpr int kFitThreads = 256;
 constexpr int kSolveThreads = 256;
 constexpr unsigned kFitNotPosDef = 0x20u;   // status bit: a system was not positive definite
-constexpr unsigned kFitSolvedDouble = 0x40u;   // status bit: ill-conditioned systems were solved in pairs of floats
+constexpr unsigned kFitSolvedAgain = 0x40u;    // status bit: ill-conditioned systems were solved in more than fp32
 constexpr int kSmallSolve = 256;               // widest system of the blocked solve
 // The fp32 factorisation's relative error grows with cond(X^T X + lambda I) times in 2^-24;
 // systems whose pivots show a condition number above this (cond >= (max L_ii / min L_ii)^2)
-// are solved again in pairs of floats.
-constexpr float kSmallSolveMaxCond = 1e3f;
+// are solved again in pairs of floats, and those that with the channels scaled alike show one above the
+// second in double.  The second line lies where pairs and double begin to differ: with sums exact in fp32 and 256
+// unknowns, the error of an fp32 W against a 64-bit solve is 2.53e-8 in both at 3.3e3, 2.52e-8 and 2.51e-8 at
+// 1.2e4, 2.58e-8 and 2.54e-8 at 6.7e4.
+constexpr float kSmallSolveMaxCond = 1e3f, kPairSolveMaxCond = 4096.f;
 
 struct FitRows {
     void* x;      // [groups][chunk][in]
@@ -186,14 +190,16 @@ __global__ void __launch_bounds__(kFitThreads) fit_rows_kernel(const __grid_cons
 // One CTA per group g = (j*Ht + h)*2 + kv.  G: fp32 X^T X [in][in], element (r, c), c <= r, at c*in + r; C: fp32 X^T Y, column-major
 // [dt][in] (element (a, o) at o*in + a); A, Z: double scratch [in][in] and [in][dt].
 // W out: the group's [in][dt] block of W_K or W_V in the cache dtype.
+// flags: NULL, or int[groups]: only the groups marked kSolveDouble.
 template <typename T>
 __global__ void __launch_bounds__(kSolveThreads) fit_solve_kernel(const float* __restrict__ G,
                                                                   const float* __restrict__ C, double* A, double* Z,
                                                                   T* wk, T* wv, int in, int dt, double lambda,
-                                                                  unsigned* status)
+                                                                  unsigned* status, const int* flags)
 {
     __shared__ int bad;
     const int g = blockIdx.x;
+    if (flags && flags[g] != kSolveDouble) return;
     double* a = A + (size_t)g * in * in;
     double* z = Z + (size_t)g * in * dt;
     const float* gg = G + (size_t)g * in * in;
@@ -950,8 +956,9 @@ using namespace kvx;
 
 struct kvx_fitter {
     Geometry geo;
-    int* redo = nullptr;                  // [1 + groups], behind the status word: how many systems the fp32
-                                          // solve leaves to the pair solve, and each group's flag
+    int* redo = nullptr;                  // [2 + groups], behind the status word: how many systems the fp32
+                                          // solve leaves to the pair solve and that one to the double solve,
+                                          // and each group's flag
     float* factor = nullptr;              // blocks of the fp32 factors (in <= kSmallSolve)
     float* factor_pair = nullptr;         // of the pair factors, once a solve has needed them
     int device = 0, num_sms = 0;
@@ -1044,7 +1051,7 @@ extern "C" KVX_API kvx_status kvx_fit_create(const kvx_translator_desc* desc, do
     if ((f->rows_bytes && cudaMalloc(&f->rows, f->rows_bytes) != cudaSuccess) ||
         cudaMalloc(&f->sums, sums_floats(f) * sizeof(float)) != cudaSuccess ||
         cudaMalloc(&f->rope, rope_bytes) != cudaSuccess ||
-        cudaMalloc(&f->status, sizeof(int) * (2 + (size_t)f->groups)) != cudaSuccess ||
+        cudaMalloc(&f->status, sizeof(int) * (3 + (size_t)f->groups)) != cudaSuccess ||
         (in <= (size_t)kSmallSolve && cudaMalloc(&f->factor, factor_bytes<F32>(f)) != cudaSuccess)) {
         const size_t rb = f->rows_bytes;
         free_fitter(f);
@@ -1191,14 +1198,16 @@ static cudaError_t launch_solve(const kvx_fitter* f, float* factor, void* w_k, v
     const int in = f->geo.in_dim, dt = f->geo.desc.dst.head_dim;
     const float* G = f->sums;
     const float* C = f->sums + (size_t)f->groups * in * in;
-    fit_factor_kernel<S><<<f->groups, kFactorThreads, 0, s>>>(G, factor, in, f->lambda, kSmallSolveMaxCond,
-                                                              kFitNotPosDef, f->status, f->redo, f->redo + 1);
+    fit_factor_kernel<S><<<f->groups, kFactorThreads, 0, s>>>(G, factor, in, f->lambda,
+                                                              S::PL == 2 ? kPairSolveMaxCond : kSmallSolveMaxCond,
+                                                              kFitNotPosDef, f->status, f->redo, f->redo + 2);
     cudaError_t ce = cudaGetLastError();
     if (ce != cudaSuccess) return ce;
     auto smem = [](int n) { return (kTrsmStages * Blocks<S>::SZ + kTrsmWarps * S::PL * n * kTrsmCols) * sizeof(float); };
     if ((ce = smem_opt_in<fit_trsm_kernel<S, T>>((int)smem(kSmallSolve))) != cudaSuccess) return ce;
     const dim3 grid(f->groups, dt / (kTrsmWarps * kTrsmCols));   // d_t is 64, 128 or 256
-    fit_trsm_kernel<S, T><<<grid, kTrsmWarps * 32, smem(in), s>>>(C, factor, (T*)w_k, (T*)w_v, in, dt, f->redo + 1);
+    fit_trsm_kernel<S, T><<<grid, kTrsmWarps * 32, smem(in), s>>>(G, C, factor, (T*)w_k, (T*)w_v, in, dt, f->lambda,
+                                                                  f->redo + 2);
     return cudaGetLastError();
 }
 template <class S>
@@ -1208,58 +1217,71 @@ static cudaError_t launch_solve(const kvx_fitter* f, float* factor, void* w_k, v
                                          : launch_solve<S, float>(f, factor, w_k, w_v, s);
 }
 
+// The double solve: every group (flags NULL) or those marked kSolveDouble.  Scratch for the factors and the solutions:
+// the row workspace when it is large enough, else a temporary allocation (the solve is not on the translation path).
+static kvx_status solve_double(kvx_fitter* f, void* w_k, void* w_v, const int* flags, cudaStream_t s)
+{
+    const int in = f->geo.in_dim, dt = f->geo.desc.dst.head_dim;
+    const float* G = f->sums;
+    const float* C = f->sums + (size_t)f->groups * in * in;
+    const size_t need = (size_t)f->groups * in * (in + dt) * sizeof(double);
+    double* scratch = nullptr;
+    bool own = false;
+    if (f->rows && need <= f->rows_bytes) scratch = (double*)f->rows;
+    else {
+        if (cudaMalloc(&scratch, need) != cudaSuccess)
+            return fit_fail(KVX_ERR_OOM, "fit_solve: scratch allocation (%zu bytes)", need);
+        own = true;
+    }
+    double* A = scratch;
+    double* Z = scratch + (size_t)f->groups * in * in;
+    if (f->geo.desc.dtype == KVX_BF16)
+        fit_solve_kernel<__nv_bfloat16><<<f->groups, kSolveThreads, 0, s>>>(
+            G, C, A, Z, (__nv_bfloat16*)w_k, (__nv_bfloat16*)w_v, in, dt, f->lambda, f->status, flags);
+    else
+        fit_solve_kernel<float><<<f->groups, kSolveThreads, 0, s>>>(G, C, A, Z, (float*)w_k, (float*)w_v, in, dt,
+                                                                    f->lambda, f->status, flags);
+    cudaError_t ce = cudaGetLastError();
+    if (ce == cudaSuccess) ce = cudaStreamSynchronize(s);
+    if (own) cudaFree(scratch);
+    if (ce != cudaSuccess) return fit_fail(KVX_ERR_CUDA, "fit_solve: %s", cudaGetErrorString(ce));
+    return KVX_OK;
+}
+
 extern "C" KVX_API kvx_status kvx_fit_solve(kvx_fitter* f, void* w_k, void* w_v, uint32_t* status_bits, void* stream)
 {
     if (!f || !w_k || !w_v) return fit_fail(KVX_ERR_INVALID_ARG, "fit_solve: NULL argument");
-    const kvx_translator_desc& D = f->geo.desc;
-    const int in = f->geo.in_dim, dt = D.dst.head_dim;
     cudaStream_t s = (cudaStream_t)stream;
     cudaError_t ce = cudaSuccess;
-    unsigned bits[2] = {0, 0};   // status word, systems left to the pair solve
-    if (in <= kSmallSolve) {
-        if ((ce = cudaMemsetAsync(f->redo, 0, sizeof(int), s)) == cudaSuccess &&
-            (ce = launch_solve<F32>(f, f->factor, w_k, w_v, s)) == cudaSuccess &&
-            (ce = cudaMemcpyAsync(bits, f->status, sizeof bits, cudaMemcpyDeviceToHost, s)) == cudaSuccess)
-            ce = cudaStreamSynchronize(s);
-        if (ce != cudaSuccess) return fit_fail(KVX_ERR_CUDA, "fit_solve: %s", cudaGetErrorString(ce));
-        if (bits[1]) {
+    unsigned bits[3] = {0, 0, 0};   // status word, systems left to the pair solve and to the double solve
+    auto read = [&]() {
+        ce = cudaMemcpyAsync(bits, f->status, sizeof bits, cudaMemcpyDeviceToHost, s);
+        if (ce == cudaSuccess) ce = cudaStreamSynchronize(s);
+        return ce;
+    };
+    if (f->geo.in_dim <= kSmallSolve) {
+        if ((ce = cudaMemsetAsync(f->redo, 0, 2 * sizeof(int), s)) != cudaSuccess ||
+            (ce = launch_solve<F32>(f, f->factor, w_k, w_v, s)) != cudaSuccess || read() != cudaSuccess)
+            return fit_fail(KVX_ERR_CUDA, "fit_solve: %s", cudaGetErrorString(ce));
+        const bool again = bits[1] > 0;
+        if (again) {
             if (!f->factor_pair && cudaMalloc(&f->factor_pair, factor_bytes<Pair>(f)) != cudaSuccess) {
                 f->factor_pair = nullptr;
                 return fit_fail(KVX_ERR_OOM, "fit_solve: scratch allocation");
             }
-            if ((ce = launch_solve<Pair>(f, f->factor_pair, w_k, w_v, s)) == cudaSuccess &&
-                (ce = cudaMemcpyAsync(bits, f->status, sizeof bits[0], cudaMemcpyDeviceToHost, s)) == cudaSuccess)
-                ce = cudaStreamSynchronize(s);
-            if (ce != cudaSuccess) return fit_fail(KVX_ERR_CUDA, "fit_solve: %s", cudaGetErrorString(ce));
-            bits[0] |= kFitSolvedDouble;
+            if ((ce = launch_solve<Pair>(f, f->factor_pair, w_k, w_v, s)) != cudaSuccess || read() != cudaSuccess)
+                return fit_fail(KVX_ERR_CUDA, "fit_solve: %s", cudaGetErrorString(ce));
         }
+        if (bits[2]) {
+            const kvx_status st = solve_double(f, w_k, w_v, f->redo + 2, s);
+            if (st != KVX_OK) return st;
+        }
+        if (bits[2] && read() != cudaSuccess) return fit_fail(KVX_ERR_CUDA, "fit_solve: %s", cudaGetErrorString(ce));
+        if (again) bits[0] |= kFitSolvedAgain;
     } else {
-        // double scratch for the factorisation and the solutions: the row workspace when it is
-        // large enough, else a temporary allocation (the solve is not on the translation path)
-        const float* G = f->sums;
-        const float* C = f->sums + (size_t)f->groups * in * in;
-        const size_t need = (size_t)f->groups * in * (in + dt) * sizeof(double);
-        double* scratch = nullptr;
-        bool own = false;
-        if (need <= f->rows_bytes) {
-            scratch = (double*)f->rows;
-        } else {
-            if (cudaMalloc(&scratch, need) != cudaSuccess) return fit_fail(KVX_ERR_OOM, "fit_solve: scratch allocation");
-            own = true;
-        }
-        double* A = scratch;
-        double* Z = scratch + (size_t)f->groups * in * in;
-        if (D.dtype == KVX_BF16)
-            fit_solve_kernel<__nv_bfloat16><<<f->groups, kSolveThreads, 0, s>>>(
-                G, C, A, Z, (__nv_bfloat16*)w_k, (__nv_bfloat16*)w_v, in, dt, f->lambda, f->status);
-        else
-            fit_solve_kernel<float><<<f->groups, kSolveThreads, 0, s>>>(G, C, A, Z, (float*)w_k, (float*)w_v, in, dt,
-                                                                        f->lambda, f->status);
-        ce = cudaGetLastError();
-        if (ce == cudaSuccess) ce = cudaMemcpyAsync(bits, f->status, sizeof bits[0], cudaMemcpyDeviceToHost, s);
-        if (ce == cudaSuccess) ce = cudaStreamSynchronize(s);
-        if (own) cudaFree(scratch);
-        if (ce != cudaSuccess) return fit_fail(KVX_ERR_CUDA, "fit_solve: %s", cudaGetErrorString(ce));
+        const kvx_status st = solve_double(f, w_k, w_v, nullptr, s);
+        if (st != KVX_OK) return st;
+        if (read() != cudaSuccess) return fit_fail(KVX_ERR_CUDA, "fit_solve: %s", cudaGetErrorString(ce));
     }
     if (status_bits) *status_bits = bits[0];
     if (bits[0] & kFitNotPosDef)

@@ -22,7 +22,17 @@
 // unevaluated sums h + l of two floats (about 48 bits), products exact by FMA (Dekker's two-product) and
 // sums by Knuth's two-sum, for the others: GB300 runs 64 fp32 FMAs for one fp64 FMA, so the twelve
 // fp32 operations of a pair multiply-add cost a fifth of one fp64 FMA.
+//
+// Pair systems are scaled first: S (X^T X + lambda I) S, S^-1 W and S X^T Y with powers of two that bring the
+// diagonal into [1/2, 2), and every right-hand side to a largest element in [1, 2).  The scaling is exact, and a
+// Cholesky solve's rounding errors do not depend on it, but the low words of a pair keep their bits only above 2^-102,
+// so without it systems of small sums (channels of 1e-16 and below) would fall back to fp32.  It also makes the
+// pivots show what the pairs have to resolve: channel scales do not count, nearly dependent channels do.
+// Where the scaled pivots show a condition number above 4096 (max_cond) 48 bits no longer leave W's error to the
+// rounding of its elements, and the system goes to the double kernel.
 #pragma once
+
+#include <climits>
 
 #include "kvx_common.cuh"
 
@@ -137,6 +147,14 @@ struct Blocks {
 };
 constexpr int kPlane = kSolveBlk * kSolveBlk;
 
+// Exponent of unknown r's scaling factor, from the diagonal of its system (Pair).
+__device__ __forceinline__ int scale_exponent(float g_rr, double lambda)
+{
+    const double d = (double)g_rr + lambda;
+    if (!(d > 0.0) || isinf(d)) return 0;
+    return -((ilogb(d) + 1) >> 1);   // d 2^(2e) in [1/2, 2)
+}
+
 // Four consecutive values of a block.
 template <class S>
 __device__ __forceinline__ void load4(const float* p, S (&x)[4])
@@ -155,10 +173,11 @@ __device__ __forceinline__ void store4(float* p, const S (&x)[4])
     if constexpr (S::PL == 2) *reinterpret_cast<float4*>(p + kPlane) = make_float4(x[0].l, x[1].l, x[2].l, x[3].l);
 }
 
-// flags[g]: 0 solved here, kSolveRedo ill-conditioned (left to the Pair kernels), kSolveBad not
-// positive definite (W is zero).  The F32 pass writes every flag and counts the redo groups in
-// *n_redo; the Pair pass (redo) works on the kSolveRedo groups only.
-constexpr int kSolveRedo = 1, kSolveBad = 2;
+// flags[g]: 0 solved here, kSolveRedo ill-conditioned (left to the Pair kernels), kSolveDouble left to the
+// double kernel, kSolveBad not positive definite (W is zero).  The F32 pass writes every flag and counts the
+// redo groups in counts[0]; the Pair pass works on the kSolveRedo groups only, and passes those that 48 bits
+// do not do on to the double kernel, counted in counts[1].
+constexpr int kSolveRedo = 1, kSolveBad = 2, kSolveDouble = 3;
 
 // acc -= A B^T over one 32 x 32 block pair; a, b: this lane's first row and column of blocks stored
 // (r, p) at p * 32 + r.
@@ -181,7 +200,7 @@ __device__ __forceinline__ void block_product(S (&acc)[8][4], const float* a, co
 template <class S>
 __global__ void __launch_bounds__(kFactorThreads, 2) fit_factor_kernel(const float* G, float* scratch, int in, double lambda,
                                                                        float max_cond, unsigned bad_bit, unsigned* status,
-                                                                       int* n_redo, int* flags)
+                                                                       int* counts, int* flags)
 {
     constexpr bool kRedo = S::PL == 2;
     constexpr int kPitch = kSolveBlk + 1, kArea = kSolveBlk * kPitch, kWarps = kFactorThreads / 32;
@@ -189,6 +208,7 @@ __global__ void __launch_bounds__(kFactorThreads, 2) fit_factor_kernel(const flo
     // before their scaling, both in place; planes kArea apart.
     __shared__ float sh[2 * S::PL * kArea];
     __shared__ float sPiv[256];
+    __shared__ int sExp[kRedo ? 256 : 1];
     __shared__ int sBad;
     float *sD = sh, *sE = sh + S::PL * kArea;
     const int g = blockIdx.x;
@@ -197,6 +217,10 @@ __global__ void __launch_bounds__(kFactorThreads, 2) fit_factor_kernel(const flo
     const Blocks<S> L{scratch + (size_t)g * solve_blocks(in) * Blocks<S>::SZ, nb};
     const float* gg = G + (size_t)g * in * in;
     if (threadIdx.x == 0) sBad = 0;
+    if (kRedo) {
+        for (int r = threadIdx.x; r < in; r += kFactorThreads) sExp[r] = scale_exponent(gg[(size_t)r * in + r], lambda);
+        __syncthreads();
+    }
     // lower blocks of X^T X: element (r, c) of the sums is at c * in + r, as in the blocks
     for (int t = warp; t < nb * (nb + 1) / 2; t += kWarps) {
         int i = 0;
@@ -208,7 +232,10 @@ __global__ void __launch_bounds__(kFactorThreads, 2) fit_factor_kernel(const flo
 #pragma unroll
         for (int c = 0; c < kSolveBlk; ++c) x[c] = from[(size_t)c * in];
 #pragma unroll
-        for (int c = 0; c < kSolveBlk; ++c) S::make(x[c]).store(f + c * kSolveBlk, kPlane);
+        for (int c = 0; c < kSolveBlk; ++c) {
+            if (kRedo) x[c] = ldexpf(x[c], sExp[i * kSolveBlk + lane] + sExp[j * kSolveBlk + c]);
+            S::make(x[c]).store(f + c * kSolveBlk, kPlane);
+        }
     }
     __syncthreads();
 
@@ -222,8 +249,9 @@ __global__ void __launch_bounds__(kFactorThreads, 2) fit_factor_kernel(const flo
                 const int c = dc + 8 * i;
                 S v = S::load(d + c * kSolveBlk + dr, kPlane);
                 if (c == dr) {
-                    v = v.add((float)lambda);
-                    if (kRedo) v = v.add((float)(lambda - (double)(float)lambda));
+                    const double l = kRedo ? ldexp(lambda, 2 * sExp[k * kSolveBlk + c]) : lambda;
+                    v = v.add((float)l);
+                    if (kRedo) v = v.add((float)(l - (double)(float)l));
                 }
                 v.store(sD + c * kPitch + dr, kArea);
                 S::make(c == dr ? 1.f : 0.f).store(sE + dr * kPitch + c, kArea);
@@ -323,13 +351,18 @@ __global__ void __launch_bounds__(kFactorThreads, 2) fit_factor_kernel(const flo
         }
         if (lane == 0) {
             const float ratio = dmax / dmin;
-            if (sBad) {
+            const bool ill = ratio * ratio > max_cond;
+            if (kRedo) {
+                if (sBad || ill) {
+                    flags[g] = kSolveDouble;
+                    atomicAdd(counts + 1, 1);
+                }
+            } else if (sBad) {
                 flags[g] = kSolveBad;
                 set_status(status, bad_bit);
-            } else if (!kRedo) {
-                const int ill = ratio * ratio > max_cond;
+            } else {
                 flags[g] = ill ? kSolveRedo : 0;
-                if (ill) atomicAdd(n_redo, 1);
+                if (ill) atomicAdd(counts, 1);
             }
         }
     }
@@ -470,21 +503,23 @@ __device__ __forceinline__ void copy16(float* dst, const float* src)
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
 }
 
-// C: X^T Y, column-major [dt][in]; W out in the cache dtype, [in][dt] per group.  dt is a multiple of the
-// CTA's kTrsmWarps * kTrsmCols columns.
+// G, C: X^T X (its diagonal, for the scaling) and X^T Y, column-major [dt][in]; W out in the cache dtype, [in][dt] per
+// group.  dt is a multiple of the CTA's kTrsmWarps * kTrsmCols columns.
 template <class S, typename T>
-__global__ void __launch_bounds__(kTrsmWarps * 32, 4) fit_trsm_kernel(const float* __restrict__ C,
+__global__ void __launch_bounds__(kTrsmWarps * 32, 4) fit_trsm_kernel(const float* __restrict__ G, const float* __restrict__ C,
                                                                       const float* __restrict__ scratch, T* wk, T* wv,
-                                                                      int in, int dt, const int* __restrict__ flags)
+                                                                      int in, int dt, double lambda,
+                                                                      const int* __restrict__ flags)
 {
     extern __shared__ float4 sm4[];   // [stage][block] | [warp][plane][in][kTrsmCols]
     constexpr bool kRedo = S::PL == 2;
+    __shared__ int sExp[kRedo ? 256 : 1];
     constexpr int SZ = Blocks<S>::SZ;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int g = blockIdx.x, o0 = (blockIdx.y * kTrsmWarps + warp) * kTrsmCols;
     const int flag = flags[g];
     T* w = ((g & 1) ? wv : wk) + (size_t)(g >> 1) * in * dt + o0;
-    if (kRedo ? flag == 0 : flag == kSolveRedo) return;
+    if (flag != (kRedo ? kSolveRedo : 0) && flag != kSolveBad) return;
     if (flag == kSolveBad) {
         for (int i = lane; i < in * kTrsmCols; i += 32)
             w[(size_t)(i / kTrsmCols) * dt + i % kTrsmCols] = from_f32<T>(0.f);
@@ -513,8 +548,39 @@ __global__ void __launch_bounds__(kTrsmWarps * 32, 4) fit_trsm_kernel(const floa
     };
     for (int i = 0; i < kTrsmStages - 1; ++i) fetch();
     const float* cc = C + ((size_t)g * dt + o0) * in;
-    for (int c = 0; c < kTrsmCols; ++c)
-        for (int r = lane; r < in; r += 32) S::make(cc[(size_t)c * in + r]).store(z + r * kTrsmCols + c, zplane);
+    int sc[kTrsmCols];   // exponents of the right-hand sides' scaling
+    if constexpr (kRedo) {
+        for (int r = threadIdx.x; r < in; r += kTrsmWarps * 32)
+            sExp[r] = scale_exponent(G[(size_t)g * in * in + (size_t)r * in + r], lambda);
+        for (int r = lane; r < in; r += 32) {   // all columns' loads in flight
+            float x[kTrsmCols];
+#pragma unroll
+            for (int c = 0; c < kTrsmCols; ++c) x[c] = cc[(size_t)c * in + r];
+#pragma unroll
+            for (int c = 0; c < kTrsmCols; ++c) z[r * kTrsmCols + c] = x[c];
+        }
+        __syncthreads();
+#pragma unroll
+        for (int c = 0; c < kTrsmCols; ++c) sc[c] = INT_MIN;
+        for (int r = lane; r < in; r += 32)
+#pragma unroll
+            for (int c = 0; c < kTrsmCols; ++c) {
+                const int e = (int)(__float_as_uint(z[r * kTrsmCols + c]) >> 23 & 0xffu);   // (subnormals: 0)
+                if (z[r * kTrsmCols + c] != 0.f && e != 255) sc[c] = max(sc[c], e - 127 + sExp[r]);
+            }
+#pragma unroll
+        for (int c = 0; c < kTrsmCols; ++c) {
+            sc[c] = __reduce_max_sync(0xffffffffu, sc[c]);
+            sc[c] = sc[c] == INT_MIN ? 0 : -sc[c];
+        }
+        for (int r = lane; r < in; r += 32)
+#pragma unroll
+            for (int c = 0; c < kTrsmCols; ++c)
+                S::make(ldexpf(z[r * kTrsmCols + c], sExp[r] + sc[c])).store(z + r * kTrsmCols + c, zplane);
+    } else {
+        for (int c = 0; c < kTrsmCols; ++c)
+            for (int r = lane; r < in; r += 32) S::make(cc[(size_t)c * in + r]).store(z + r * kTrsmCols + c, zplane);
+    }
     __syncwarp();
     int n = 0;
     // the next block: landed for every thread, the one before it free for the fetch after next
@@ -548,8 +614,11 @@ __global__ void __launch_bounds__(kTrsmWarps * 32, 4) fit_trsm_kernel(const floa
         }
     for (int r = lane; r < in; r += 32)
 #pragma unroll
-        for (int c = 0; c < kTrsmCols; ++c)
-            w[(size_t)r * dt + c] = from_f32<T>(S::load(z + r * kTrsmCols + c, zplane).value());
+        for (int c = 0; c < kTrsmCols; ++c) {
+            float x = S::load(z + r * kTrsmCols + c, zplane).value();
+            if constexpr (kRedo) x = ldexpf(x, sExp[r] - sc[c]);
+            w[(size_t)r * dt + c] = from_f32<T>(x);
+        }
 }
 
 }  // namespace

@@ -336,6 +336,44 @@ def test_blocked_solve_sizes_match_a_double_solve(ds, kl, dt, spread):
             assert _rel(got, ref) <= 16 * (T + 4 * n_in) * 2.0 ** -24, (kv, j, _rel(got, ref))
 
 
+def _solve_64(G, C):
+    """W of G W = C: a double factor refined with long double residuals, the unknowns scaled alike by powers of two."""
+    d = 2.0 ** -np.round(np.log2(np.sqrt(np.diag(G))))
+    Gs, Cs = (G * d[:, None] * d).astype(np.longdouble), (C * d[:, None]).astype(np.longdouble)
+    L = np.linalg.cholesky(Gs.astype(np.float64))
+    W = np.zeros_like(Cs)
+    for _ in range(6):
+        R = (Cs - Gs @ W).astype(np.float64)
+        W = W + np.linalg.solve(L.T, np.linalg.solve(L, R))
+    return (W * d[:, None]).astype(np.float64), np.linalg.cond(Gs.astype(np.float64))
+
+
+@pytest.mark.parametrize("sx,sy", [(1.0, 1.0), (2.0 ** -62, 1.0), (2.0 ** -62, 2.0 ** -50), (2.0 ** 40, 2.0 ** -30)])
+@pytest.mark.parametrize("spread", [False, True])
+@pytest.mark.parametrize("density", [0.5, 0.1, 0.02])
+def test_ill_conditioned_solves_are_exact_to_the_rounding_of_w(density, spread, sx, sy):
+    """The second head's channels are the first's plus sparse steps of one (scaled condition numbers of 1e4 to 4e5);
+    spread: channel scales over seven powers of two; sx, sy: caches of any magnitude.  Entries are small integers
+    times powers of two, so every sum is exact in fp32 and only the solve's error and W's rounding (2^-24 an
+    element) remain: pairs below a scaled condition number of about 4096 (by the pivots; 3e4 by the eigenvalues),
+    whose 2^-46 an operation adds no more than cond 2^-44, and double above."""
+    rng = np.random.default_rng(7)
+    T, h, dt = 2000, 64, 64
+    a = rng.integers(-40, 41, size=(T, h))
+    X = np.concatenate([a, a + rng.choice([-1, 1], size=(T, h)) * (rng.random((T, h)) < density)], 1).astype(np.float64)
+    X *= sx * (2.0 ** -rng.integers(0, 8, size=2 * h) if spread else 1.0)
+    Y = rng.integers(-40, 41, size=(T, dt)) * sy
+    cache = lambda x: torch.from_numpy(x.astype(np.float32)).cuda().view(1, 1, T, -1)
+    f = kvx.Fitter(synth.ModelGeom(1, 1, 2 * h, 0.0), synth.ModelGeom(1, 1, dt, 0.0), 0.0, layer_map=[0], dtype=kvx.KVX_FP32)
+    i32 = lambda x: torch.tensor(x, dtype=torch.int32, device="cuda")
+    f.accumulate([cache(X)], [cache(X)], i32([T]), i32([0, T]), T, [cache(Y)], [cache(Y)])
+    w = [torch.zeros((1, 1, 2 * h, dt), device="cuda") for _ in range(2)]
+    assert f.solve(w[0], w[1]) == 0x40
+    ref, cond = _solve_64(X.T @ X, X.T @ Y)
+    for got in w:
+        assert _rel(got[0, 0].cpu().numpy(), ref) <= 2.0 ** -24 + min(cond, 3e4) * 2.0 ** -44, (_rel(got[0, 0].cpu().numpy(), ref), cond)
+
+
 def test_wide_systems_from_tensor_core_sums_match_a_double_solve():
     """384 unknowns (three source layers of 128 channels): three row blocks of tensor-core sums, solved in
     double.  bf16 rows without rotation are exact inputs, so only W's rounding to bf16 (2^-9 an element)
