@@ -374,7 +374,8 @@ KVX_API kvx_status kvx_fit_accumulate(kvx_fitter* f, const kvx_src_kv* src, cons
  * the fitter's status word: KVX_DEV_* bits from the accumulation passes (rows left out), 0x20
  * when a system was not positive definite (lambda = 0 with too few tokens; its W is zero), in
  * which case the call returns KVX_ERR_DEVICE_STATUS, and 0x40 (informational) when
- * ill-conditioned systems were solved again in more than fp32.  Calls on one fitter must be ordered
+ * ill-conditioned systems, or systems whose fp32 factor broke down, were
+ * solved again in more than fp32.  Calls on one fitter must be ordered
  * (one stream, or synchronised by the caller). */
 KVX_API kvx_status kvx_fit_solve(kvx_fitter* f, void* w_k, void* w_v, uint32_t* status_bits, void* stream);
 

@@ -190,16 +190,19 @@ __global__ void __launch_bounds__(kFitThreads) fit_rows_kernel(const __grid_cons
 // One CTA per group g = (j*Ht + h)*2 + kv.  G: fp32 X^T X [in][in], element (r, c), c <= r, at c*in + r; C: fp32 X^T Y, column-major
 // [dt][in] (element (a, o) at o*in + a); A, Z: double scratch [in][in] and [in][dt].
 // W out: the group's [in][dt] block of W_K or W_V in the cache dtype.
-// flags: NULL, or int[groups]: only the groups marked kSolveDouble.
+// flags: NULL, or int[groups]: only the groups marked kSolveDouble or kSolveBroken.  The latter, whose fp32 factor
+// broke down, have pivots within the rounding of exact zeros to tell from positive ones: a pivot counts as positive
+// above in 2^-50 of its diagonal element.  solved: counts those of them that are solved.
 template <typename T>
 __global__ void __launch_bounds__(kSolveThreads) fit_solve_kernel(const float* __restrict__ G,
                                                                   const float* __restrict__ C, double* A, double* Z,
                                                                   T* wk, T* wv, int in, int dt, double lambda,
-                                                                  unsigned* status, const int* flags)
+                                                                  unsigned* status, const int* flags, int* solved)
 {
     __shared__ int bad;
     const int g = blockIdx.x;
-    if (flags && flags[g] != kSolveDouble) return;
+    if (flags && flags[g] != kSolveDouble && flags[g] != kSolveBroken) return;
+    const double tiny = flags && flags[g] == kSolveBroken ? in * 0x1p-50 : 0.0;
     double* a = A + (size_t)g * in * in;
     double* z = Z + (size_t)g * in * dt;
     const float* gg = G + (size_t)g * in * in;
@@ -214,7 +217,8 @@ __global__ void __launch_bounds__(kSolveThreads) fit_solve_kernel(const float* _
     for (int k = 0; k < in; ++k) {
         if (threadIdx.x == 0) {
             double d = a[(size_t)k * in + k];
-            if (!(d > 0.0)) { bad = 1; d = 1.0; }
+            const double zero = tiny > 0.0 ? tiny * ((double)gg[(size_t)k * in + k] + lambda) : 0.0;
+            if (!(d > zero)) { bad = 1; d = 1.0; }
             a[(size_t)k * in + k] = sqrt(d);
         }
         __syncthreads();
@@ -245,7 +249,10 @@ __global__ void __launch_bounds__(kSolveThreads) fit_solve_kernel(const float* _
     T* w = (g & 1) ? wv : wk;
     const size_t off = (size_t)(g >> 1) * in * dt;   // (j*Ht + h) block of [Lt][Ht][in][dt]
     for (int i = threadIdx.x; i < in * dt; i += blockDim.x) w[off + i] = from_f32<T>(bad ? 0.f : (float)z[i]);
-    if (bad && threadIdx.x == 0) set_status(status, kFitNotPosDef);
+    if (threadIdx.x == 0) {
+        if (bad) set_status(status, kFitNotPosDef);
+        else if (flags && flags[g] == kSolveBroken) atomicAdd(solved, 1);
+    }
 }
 
 // ------------------------------------------------------------------ Gram sums on the CUDA cores
@@ -956,9 +963,9 @@ using namespace kvx;
 
 struct kvx_fitter {
     Geometry geo;
-    int* redo = nullptr;                  // [2 + groups], behind the status word: how many systems the fp32
-                                          // solve leaves to the pair solve and that one to the double solve,
-                                          // and each group's flag
+    int* redo = nullptr;                  // [3 + groups], behind the status word: how many systems go to the
+                                          // pair solve, to the double solve, and were solved by it after their
+                                          // fp32 factor broke down; each group's flag
     float* factor = nullptr;              // blocks of the fp32 factors (in <= kSmallSolve)
     float* factor_pair = nullptr;         // of the pair factors, once a solve has needed them
     int device = 0, num_sms = 0;
@@ -1051,7 +1058,7 @@ extern "C" KVX_API kvx_status kvx_fit_create(const kvx_translator_desc* desc, do
     if ((f->rows_bytes && cudaMalloc(&f->rows, f->rows_bytes) != cudaSuccess) ||
         cudaMalloc(&f->sums, sums_floats(f) * sizeof(float)) != cudaSuccess ||
         cudaMalloc(&f->rope, rope_bytes) != cudaSuccess ||
-        cudaMalloc(&f->status, sizeof(int) * (3 + (size_t)f->groups)) != cudaSuccess ||
+        cudaMalloc(&f->status, sizeof(int) * (4 + (size_t)f->groups)) != cudaSuccess ||
         (in <= (size_t)kSmallSolve && cudaMalloc(&f->factor, factor_bytes<F32>(f)) != cudaSuccess)) {
         const size_t rb = f->rows_bytes;
         free_fitter(f);
@@ -1200,14 +1207,14 @@ static cudaError_t launch_solve(const kvx_fitter* f, float* factor, void* w_k, v
     const float* C = f->sums + (size_t)f->groups * in * in;
     fit_factor_kernel<S><<<f->groups, kFactorThreads, 0, s>>>(G, factor, in, f->lambda,
                                                               S::PL == 2 ? kPairSolveMaxCond : kSmallSolveMaxCond,
-                                                              kFitNotPosDef, f->status, f->redo, f->redo + 2);
+                                                              f->redo, f->redo + 3);
     cudaError_t ce = cudaGetLastError();
     if (ce != cudaSuccess) return ce;
     auto smem = [](int n) { return (kTrsmStages * Blocks<S>::SZ + kTrsmWarps * S::PL * n * kTrsmCols) * sizeof(float); };
     if ((ce = smem_opt_in<fit_trsm_kernel<S, T>>((int)smem(kSmallSolve))) != cudaSuccess) return ce;
     const dim3 grid(f->groups, dt / (kTrsmWarps * kTrsmCols));   // d_t is 64, 128 or 256
     fit_trsm_kernel<S, T><<<grid, kTrsmWarps * 32, smem(in), s>>>(G, C, factor, (T*)w_k, (T*)w_v, in, dt, f->lambda,
-                                                                  f->redo + 2);
+                                                                  f->redo + 3);
     return cudaGetLastError();
 }
 template <class S>
@@ -1237,10 +1244,10 @@ static kvx_status solve_double(kvx_fitter* f, void* w_k, void* w_v, const int* f
     double* Z = scratch + (size_t)f->groups * in * in;
     if (f->geo.desc.dtype == KVX_BF16)
         fit_solve_kernel<__nv_bfloat16><<<f->groups, kSolveThreads, 0, s>>>(
-            G, C, A, Z, (__nv_bfloat16*)w_k, (__nv_bfloat16*)w_v, in, dt, f->lambda, f->status, flags);
+            G, C, A, Z, (__nv_bfloat16*)w_k, (__nv_bfloat16*)w_v, in, dt, f->lambda, f->status, flags, f->redo + 2);
     else
         fit_solve_kernel<float><<<f->groups, kSolveThreads, 0, s>>>(G, C, A, Z, (float*)w_k, (float*)w_v, in, dt,
-                                                                    f->lambda, f->status, flags);
+                                                                    f->lambda, f->status, flags, f->redo + 2);
     cudaError_t ce = cudaGetLastError();
     if (ce == cudaSuccess) ce = cudaStreamSynchronize(s);
     if (own) cudaFree(scratch);
@@ -1253,18 +1260,17 @@ extern "C" KVX_API kvx_status kvx_fit_solve(kvx_fitter* f, void* w_k, void* w_v,
     if (!f || !w_k || !w_v) return fit_fail(KVX_ERR_INVALID_ARG, "fit_solve: NULL argument");
     cudaStream_t s = (cudaStream_t)stream;
     cudaError_t ce = cudaSuccess;
-    unsigned bits[3] = {0, 0, 0};   // status word, systems left to the pair solve and to the double solve
+    unsigned bits[4] = {0, 0, 0, 0};   // status word and the counts behind it
     auto read = [&]() {
         ce = cudaMemcpyAsync(bits, f->status, sizeof bits, cudaMemcpyDeviceToHost, s);
         if (ce == cudaSuccess) ce = cudaStreamSynchronize(s);
         return ce;
     };
     if (f->geo.in_dim <= kSmallSolve) {
-        if ((ce = cudaMemsetAsync(f->redo, 0, 2 * sizeof(int), s)) != cudaSuccess ||
+        if ((ce = cudaMemsetAsync(f->redo, 0, 3 * sizeof(int), s)) != cudaSuccess ||
             (ce = launch_solve<F32>(f, f->factor, w_k, w_v, s)) != cudaSuccess || read() != cudaSuccess)
             return fit_fail(KVX_ERR_CUDA, "fit_solve: %s", cudaGetErrorString(ce));
-        const bool again = bits[1] > 0;
-        if (again) {
+        if (bits[1]) {
             if (!f->factor_pair && cudaMalloc(&f->factor_pair, factor_bytes<Pair>(f)) != cudaSuccess) {
                 f->factor_pair = nullptr;
                 return fit_fail(KVX_ERR_OOM, "fit_solve: scratch allocation");
@@ -1273,11 +1279,11 @@ extern "C" KVX_API kvx_status kvx_fit_solve(kvx_fitter* f, void* w_k, void* w_v,
                 return fit_fail(KVX_ERR_CUDA, "fit_solve: %s", cudaGetErrorString(ce));
         }
         if (bits[2]) {
-            const kvx_status st = solve_double(f, w_k, w_v, f->redo + 2, s);
+            const kvx_status st = solve_double(f, w_k, w_v, f->redo + 3, s);
             if (st != KVX_OK) return st;
+            if (read() != cudaSuccess) return fit_fail(KVX_ERR_CUDA, "fit_solve: %s", cudaGetErrorString(ce));
         }
-        if (bits[2] && read() != cudaSuccess) return fit_fail(KVX_ERR_CUDA, "fit_solve: %s", cudaGetErrorString(ce));
-        if (again) bits[0] |= kFitSolvedAgain;
+        if (bits[1] || bits[3]) bits[0] |= kFitSolvedAgain;
     } else {
         const kvx_status st = solve_double(f, w_k, w_v, nullptr, s);
         if (st != KVX_OK) return st;

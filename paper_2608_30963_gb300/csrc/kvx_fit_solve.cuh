@@ -174,10 +174,10 @@ __device__ __forceinline__ void store4(float* p, const S (&x)[4])
 }
 
 // flags[g]: 0 solved here, kSolveRedo ill-conditioned (left to the Pair kernels), kSolveDouble left to the
-// double kernel, kSolveBad not positive definite (W is zero).  The F32 pass writes every flag and counts the
-// redo groups in counts[0]; the Pair pass works on the kSolveRedo groups only, and passes those that 48 bits
-// do not do on to the double kernel, counted in counts[1].
-constexpr int kSolveRedo = 1, kSolveBad = 2, kSolveDouble = 3;
+// double kernel, kSolveBroken too: a pivot was not positive.  The F32 pass writes every flag and counts the redo
+// groups in counts[0]; the Pair pass works on those only.  What either leaves to the double kernel is counted in
+// counts[1]; that kernel alone declares a system not positive definite.
+constexpr int kSolveRedo = 1, kSolveDouble = 2, kSolveBroken = 3;
 
 // acc -= A B^T over one 32 x 32 block pair; a, b: this lane's first row and column of blocks stored
 // (r, p) at p * 32 + r.
@@ -199,8 +199,7 @@ __device__ __forceinline__ void block_product(S (&acc)[8][4], const float* a, co
 
 template <class S>
 __global__ void __launch_bounds__(kFactorThreads, 2) fit_factor_kernel(const float* G, float* scratch, int in, double lambda,
-                                                                       float max_cond, unsigned bad_bit, unsigned* status,
-                                                                       int* counts, int* flags)
+                                                                       float max_cond, int* counts, int* flags)
 {
     constexpr bool kRedo = S::PL == 2;
     constexpr int kPitch = kSolveBlk + 1, kArea = kSolveBlk * kPitch, kWarps = kFactorThreads / 32;
@@ -352,15 +351,11 @@ __global__ void __launch_bounds__(kFactorThreads, 2) fit_factor_kernel(const flo
         if (lane == 0) {
             const float ratio = dmax / dmin;
             const bool ill = ratio * ratio > max_cond;
-            if (kRedo) {
-                if (sBad || ill) {
-                    flags[g] = kSolveDouble;
-                    atomicAdd(counts + 1, 1);
-                }
-            } else if (sBad) {
-                flags[g] = kSolveBad;
-                set_status(status, bad_bit);
-            } else {
+            const int to_double = sBad ? kSolveBroken : kRedo && ill ? kSolveDouble : 0;
+            if (to_double) {
+                flags[g] = to_double;
+                atomicAdd(counts + 1, 1);
+            } else if (!kRedo) {
                 flags[g] = ill ? kSolveRedo : 0;
                 if (ill) atomicAdd(counts, 1);
             }
@@ -517,14 +512,8 @@ __global__ void __launch_bounds__(kTrsmWarps * 32, 4) fit_trsm_kernel(const floa
     constexpr int SZ = Blocks<S>::SZ;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int g = blockIdx.x, o0 = (blockIdx.y * kTrsmWarps + warp) * kTrsmCols;
-    const int flag = flags[g];
     T* w = ((g & 1) ? wv : wk) + (size_t)(g >> 1) * in * dt + o0;
-    if (flag != (kRedo ? kSolveRedo : 0) && flag != kSolveBad) return;
-    if (flag == kSolveBad) {
-        for (int i = lane; i < in * kTrsmCols; i += 32)
-            w[(size_t)(i / kTrsmCols) * dt + i % kTrsmCols] = from_f32<T>(0.f);
-        return;
-    }
+    if (flags[g] != (kRedo ? kSolveRedo : 0)) return;
     const int nb = in / kSolveBlk, zplane = in * kTrsmCols;
     float* stage = reinterpret_cast<float*>(sm4);
     float* z = stage + kTrsmStages * SZ + (size_t)warp * S::PL * zplane;

@@ -374,6 +374,37 @@ def test_ill_conditioned_solves_are_exact_to_the_rounding_of_w(density, spread, 
         assert _rel(got[0, 0].cpu().numpy(), ref) <= 2.0 ** -24 + min(cond, 3e4) * 2.0 ** -44, (_rel(got[0, 0].cpu().numpy(), ref), cond)
 
 
+@pytest.mark.parametrize("kind", ["nearly_singular", "singular", "too_few_tokens"])
+def test_only_systems_that_double_cannot_factor_are_refused(kind):
+    """Sums exact in fp32.  nearly_singular: the second head's channels are the first's plus one step in one token, a
+    last pivot of about 2e-7 of its diagonal element, below what 128 fp32 elimination steps resolve (2^-24 each):
+    the fp32 factor breaks down, the system is positive definite, and W comes out to its rounding.  singular: the
+    heads coincide; too_few_tokens: 100 of 128.  Those are refused, with W zero."""
+    rng = np.random.default_rng(11)
+    T, h, dt = (100 if kind == "too_few_tokens" else 2000), 64, 64
+    a = rng.integers(-90, 91, size=(T, h))
+    b = a.copy()
+    if kind == "nearly_singular":
+        b[rng.permutation(T)[:h], np.arange(h)] += 1
+    elif kind == "too_few_tokens":
+        b = rng.integers(-90, 91, size=(T, h))
+    X, Y = np.concatenate([a, b], 1).astype(np.float64), rng.integers(-40, 41, size=(T, dt)).astype(np.float64)
+    assert (X * X).sum(0).max() < 2 ** 24
+    cache = lambda x: torch.from_numpy(x.astype(np.float32)).cuda().view(1, 1, T, -1)
+    f = kvx.Fitter(synth.ModelGeom(1, 1, 2 * h, 0.0), synth.ModelGeom(1, 1, dt, 0.0), 0.0, layer_map=[0], dtype=kvx.KVX_FP32)
+    i32 = lambda x: torch.tensor(x, dtype=torch.int32, device="cuda")
+    f.accumulate([cache(X)], [cache(X)], i32([T]), i32([0, T]), T, [cache(Y)], [cache(Y)])
+    w = [torch.full((1, 1, 2 * h, dt), float("nan"), device="cuda") for _ in range(2)]
+    bits = f.solve(w[0], w[1])
+    if kind != "nearly_singular":
+        assert bits & ~0x40 == 0x20 and all(bool((x == 0).all()) for x in w), hex(bits)
+        return
+    assert bits == 0x40, hex(bits)
+    ref, cond = _solve_64(X.T @ X, X.T @ Y)
+    for got in w:
+        assert _rel(got[0, 0].cpu().numpy(), ref) <= 2.0 ** -24 + cond * 2.0 ** -46, (_rel(got[0, 0].cpu().numpy(), ref), cond)
+
+
 def test_wide_systems_from_tensor_core_sums_match_a_double_solve():
     """384 unknowns (three source layers of 128 channels): three row blocks of tensor-core sums, solved in
     double.  bf16 rows without rotation are exact inputs, so only W's rounding to bf16 (2^-9 an element)
