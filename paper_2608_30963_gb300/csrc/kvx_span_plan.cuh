@@ -35,8 +35,7 @@ __device__ __forceinline__ int2 load_span(const TranslateParams& P, int tp)
 }
 
 // Source-side resolution of one target token (sequence, clamped span) from its
-// loaded span bounds.  FLAG: report what was clamped in the status word.
-template <bool FLAG>
+// loaded span bounds; what was clamped is reported in the status word.
 __device__ __forceinline__ void resolve_src(const TranslateParams& P, const SeqView& sv, int tp, int2 span, int& b,
                                             int& lo, int& hi)
 {
@@ -44,13 +43,13 @@ __device__ __forceinline__ void resolve_src(const TranslateParams& P, const SeqV
     const int t = tp - sv.off[b];
     int S = sv.slen[b];
     if (S > P.src_max_seq || S < 0) {
-        if (FLAG) set_status(P.status, KVX_DEV_SEQ_CLAMPED);
+        set_status(P.status, KVX_DEV_SEQ_CLAMPED);
         S = S < 0 ? 0 : P.src_max_seq;
     }
     if (P.span_lo) { lo = span.x; hi = span.y; }
     else { lo = t; hi = t + 1; }
     if (lo < 0 || hi > S || hi <= lo) {
-        if (FLAG) set_status(P.status, KVX_DEV_SPAN_CLAMPED);
+        set_status(P.status, KVX_DEV_SPAN_CLAMPED);
         lo = lo < 0 ? 0 : (lo > S - 1 ? S - 1 : lo);
         hi = hi > S ? S : hi;
         if (hi <= lo) hi = lo + 1;

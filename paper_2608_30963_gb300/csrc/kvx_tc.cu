@@ -39,7 +39,7 @@ __global__ void __launch_bounds__(128) span_plan_kernel(const __grid_constant__ 
     const int tp = t_begin + sub * kSub + lane;
     const bool valid = tp < t_end;
     int b = -1, lo = 0, hi = 0;
-    if (valid) resolve_src<true>(P, sv, tp, load_span(P, tp), b, lo, hi);
+    if (valid) resolve_src(P, sv, tp, load_span(P, tp), b, lo, hi);
     write_window_plan(valid, b, lo, hi, sub, lane, cap_rows, hdr, ent);
 }
 

@@ -780,7 +780,7 @@ __global__ void __launch_bounds__(kTileM) span_rows_kernel(const __grid_constant
     const int tp = t_begin + (int)blockIdx.x * kTileM + (int)threadIdx.x;
     const bool valid = tp < t_end;
     int b = -1, lo = 0, hi = 0;
-    if (valid) resolve_src<true>(P, sv, tp, load_span(P, tp), b, lo, hi);
+    if (valid) resolve_src(P, sv, tp, load_span(P, tp), b, lo, hi);
     const bool inwin = write_window_plan(valid, b, lo, hi, (int)blockIdx.x * (kTileM / 32) + warp, lane, cap_rows, hdr, win);
     const int n = valid ? hi - lo : -1;
     // (a tile's sums are at most 128 x 2048 = kRowsMax)
