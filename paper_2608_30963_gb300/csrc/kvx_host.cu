@@ -499,7 +499,7 @@ static kvx_status translate_impl(kvx_translator* tr, const kvx_src_kv* src, cons
                                  &tr->last_launches);
         tr->last_span_tokens = P.T_total;
     } else {
-        ce = launch_translate_simt(P, D.dtype, (cudaStream_t)stream);
+        ce = launch_translate_simt(P, tr->num_sms, D.dtype, (cudaStream_t)stream);
         tr->last_launches = 1;
     }
     if (ce != cudaSuccess) return fail(KVX_ERR_CUDA, "translate: launch failed: %s", cudaGetErrorString(ce));

@@ -6,8 +6,10 @@
 namespace kvx {
 struct TranslateParams;
 
+constexpr int kSimtThreads = 128;   // threads of a CTA of the CUDA-core kernel
+// its dynamic shared memory, for the larger of its tiles that fits
 size_t simt_smem_bytes(int in_dim, int dt);
-cudaError_t launch_translate_simt(const TranslateParams& P, int dtype, cudaStream_t stream);
+cudaError_t launch_translate_simt(const TranslateParams& P, int num_sms, int dtype, cudaStream_t stream);
 // W = A . B for n (layer, head, K|V) matrices (latent adapters, at translator creation)
 cudaError_t launch_fold_low_rank(const void* a, const void* b, void* w, int n, int in_dim, int rank, int out,
                                  int dtype, cudaStream_t stream);

@@ -34,6 +34,7 @@ std::mutex g_setup_mutex;
 // address belongs to that context, so a call under another context (a non-primary one, or the
 // primary context re-created after cudaDeviceReset) looks it up again.
 unsigned char* g_scratch_addr[kMaxDevices];
+int g_num_sms[kMaxDevices];
 void* g_scratch_ctx[kMaxDevices];
 
 // The calling thread's current driver context (NULL if it cannot be read).
@@ -151,11 +152,12 @@ extern "C" KVX_API kvx_status kvx_translate_static(const kvx_translator_desc* de
         return fail(KVX_ERR_INVALID_ARG, "translate_static: bad page table");
     }
 
-    // once per device, with that device current: the device address of the scratch array
+    // once per device, with that device current: the device address of the scratch array, and the SM count
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices)
         return fail(KVX_ERR_CUDA, "translate_static: no usable current device");
     unsigned char* scratch = nullptr;
+    int num_sms = 0;
     {
         std::lock_guard<std::mutex> lock(g_setup_mutex);
         void* ctx = current_context();
@@ -164,10 +166,14 @@ extern "C" KVX_API kvx_status kvx_translate_static(const kvx_translator_desc* de
             const cudaError_t ce = cudaGetSymbolAddress(&ptr, g_static_scratch);
             if (ce != cudaSuccess || !ptr)
                 return fail(KVX_ERR_CUDA, "translate_static: cudaGetSymbolAddress: %s", cudaGetErrorString(ce));
+            const cudaError_t ae = cudaDeviceGetAttribute(&g_num_sms[dev], cudaDevAttrMultiProcessorCount, dev);
+            if (ae != cudaSuccess)
+                return fail(KVX_ERR_CUDA, "translate_static: cudaDeviceGetAttribute: %s", cudaGetErrorString(ae));
             g_scratch_addr[dev] = (unsigned char*)ptr;
             g_scratch_ctx[dev] = current_context();   // the lookup made the runtime's context current
         }
         scratch = g_scratch_addr[dev];
+        num_sms = g_num_sms[dev];
     }
     cudaStream_t st = (cudaStream_t)stream;
     unsigned* status = (unsigned*)scratch;
@@ -211,7 +217,7 @@ extern "C" KVX_API kvx_status kvx_translate_static(const kvx_translator_desc* de
             if (!P.src_k[j] || !P.src_v[j] || !P.dst_k[j] || !P.dst_v[j])
                 return fail(KVX_ERR_INVALID_ARG, "translate_static: NULL cache pointer for target layer %d", j);
         }
-        if ((ce = launch_translate_simt(P, desc->dtype, st)) != cudaSuccess)
+        if ((ce = launch_translate_simt(P, num_sms, desc->dtype, st)) != cudaSuccess)
             return fail(KVX_ERR_CUDA, "translate_static: launch failed: %s", cudaGetErrorString(ce));
     }
     if (status_bits) {

@@ -1,4 +1,5 @@
-// kvx_schedule.h -- host-side work split of the identity-alignment kernel (no device code).
+// kvx_schedule.h -- host-side work splits: the identity-alignment kernel's shares, the CUDA-core kernel's tiles
+// (no device code).
 #pragma once
 
 #include <algorithm>
@@ -39,6 +40,15 @@ inline void pair_v_shares(int grid, long long UH, long long m_tiles, unsigned sh
     delete[] byv;
     delete[] ck;
     delete[] cv;
+}
+
+// Target tokens of one CTA of the CUDA-core kernel (kvx_simt.cu): 32 where such tiles give two CTAs an SM and their
+// input rows fit shared memory, else 16 (the measurements stand beside the launch).  per_head: CTAs of one head and
+// token tile.
+inline int simt_tile_tokens(int tokens, int heads, int per_head, int layers, bool fits32, int num_sms)
+{
+    const long long tiles = (long long)((tokens + 31) / 32) * heads * per_head * layers * 2;
+    return fits32 && tiles >= 2ll * num_sms ? 32 : 16;
 }
 
 }  // namespace kvx

@@ -12,14 +12,14 @@
 // Section 5 (T_theta per layer and KV head).
 //
 // Bound: fp32 FMA issue (128 a clock and SM).  Each output is one accumulator in ascending input
-// order.  1000 tokens of 7B -> 1.5B shapes (3.7 G FMA): 201 us; 608 us with a thread per output channel
+// order.  1000 tokens of 7B -> 1.5B shapes (3.7 G FMA): 199 us; 608 us with a thread per output channel
 // and scalar reads of A and W.
 #include "kvx_common.cuh"
 #include "kvx_kernels.h"
+#include "kvx_schedule.h"
 
 namespace kvx {
 
-constexpr int kSimtThreads = 128;
 constexpr int kSimtPad = 4;         // floats between two rows of A: 16-byte reads of two rows miss each other's banks
 constexpr int kSimtSmemMax = 200 * 1024;
 
@@ -27,7 +27,7 @@ constexpr int kSimtSmemMax = 200 * 1024;
 // thread, so 8 or 16 threads across the channels and 16 or 8 groups of tokens.
 constexpr int simt_groups(int slots) { return kSimtThreads / (slots / 4); }
 // Input rows of W per shared-memory block: 8 under 32-token tiles, which leaves room for a fifth CTA an SM
-// (201 against 210 us for the case above), 16 under 16-token tiles, whose chain of blocks counts.
+// (199 us for the case above; 16 rows and four CTAs: 210), 16 under 16-token tiles, whose chain of blocks counts.
 __host__ __device__ constexpr int simt_k(int tm) { return tm == 32 ? 8 : 16; }
 
 // 4 consecutive elements; VEC: 16-byte aligned rows, else element by element.
@@ -64,7 +64,7 @@ __device__ __forceinline__ void store4(__nv_bfloat16* p, float4 x)
     }
 }
 // (c0, c1) += x (w0, w1): one packed instruction for two fp32 FMAs, each rounded as fmaf.  The packed
-// form halves the issue slots of the projection (236 to 211 us for the case above, four CTAs an SM).
+// form halves the issue slots of the projection (the case above with four CTAs an SM: 210 us, 236 with fmaf).
 __device__ __forceinline__ void fma2(float& c0, float& c1, float x, float w0, float w1)
 {
     asm("{\n\t.reg .b64 a, b, c;\n\tmov.b64 a, {%2, %2};\n\tmov.b64 b, {%3, %4};\n\tmov.b64 c, {%0, %1};\n\t"
@@ -107,7 +107,7 @@ __global__ void __launch_bounds__(kSimtThreads) translate_simt_kernel(const __gr
     const int ntok = min(TM, P.T_total - t0);
     const int tid = threadIdx.x;
 
-    // W block b: rows [16 b, 16 b + 16), the CTA's channels, in registers until the block before is used
+    // W block b: rows [kSimtK b, kSimtK b + kSimtK), the CTA's channels, in registers until the block before is used
     const T* W = (const T*)P.w + ((size_t)(kv * P.Lt + j) * P.Ht + h) * (size_t)P.in_dim * P.dt;
     float4 wreg[WPT];
     int w_k[WPT], w_c[WPT], w_s[WPT];
@@ -321,13 +321,12 @@ size_t simt_smem_bytes(int in_dim, int dt)
     return big <= (size_t)kSimtSmemMax ? big : simt_smem(in_dim, simt_slots(dt), 16);
 }
 
-cudaError_t launch_translate_simt(const TranslateParams& P, int dtype, cudaStream_t stream)
+cudaError_t launch_translate_simt(const TranslateParams& P, int num_sms, int dtype, cudaStream_t stream)
 {
-    // 32-token tiles where they give two CTAs an SM (152 SMs) and A fits shared memory, else 16: four CTAs of
-    // 32 tokens an SM overlap their phases (211 us, with 8 rows of W a block five and 199; two of 64 tokens and 128 threads 256, of 256 threads 227),
-    // and below two CTAs an SM the chain of one CTA counts
-    const long long tiles = (long long)((P.T_total + 31) / 32) * P.Ht * (P.dt / (2 * simt_slots(P.dt))) * P.Lt * 2;
-    const bool big = tiles >= 2 * 152 && simt_smem(P.in_dim, simt_slots(P.dt), 32) <= (size_t)kSimtSmemMax;
+    // 32 or 16 tokens a CTA: five CTAs of 32 tokens an SM overlap their phases (the case at the top: 199 us; two of 64
+    // tokens and 128 threads 256, of 256 threads 227), and below two CTAs an SM the chain of one CTA counts
+    const bool big = simt_tile_tokens(P.T_total, P.Ht, P.dt / (2 * simt_slots(P.dt)), P.Lt,
+                                      simt_smem(P.in_dim, simt_slots(P.dt), 32) <= (size_t)kSimtSmemMax, num_sms) == 32;
     // the strides are whole 16-byte groups; the caches of the allocation-free entry may start anywhere
     uintptr_t a = 0;
     for (int i = 0; i < P.Lt * P.kl; ++i) a |= (uintptr_t)P.src_k[i] | (uintptr_t)P.src_v[i];

@@ -4,8 +4,9 @@
 //   freq <d> <rotary_dim> <type> <factor> <low> <high> <orig> <base> then d/2 lines "<i> <f_i>"
 //   ok <1|0>                                                  -- rope_schedule_ok
 //   vshares <grid> then grid lines "<cta> <v share>"           -- pair_v_shares
+//   tile <tokens>                                             -- simt_tile_tokens
 // for the cases read from standard input (one per line, same fields; vshares reads
-// <grid> <units per K|V> <units per group>).
+// <grid> <units per K|V> <units per group>, tile <tokens> <heads> <CTAs a head> <layers> <fits> <SMs>).
 #include <cstdio>
 #include <cstring>
 
@@ -47,6 +48,10 @@ int main()
             kvx::pair_v_shares(grid, uh, mt, v);
             std::printf("vshares %d\n", grid);
             for (int c = 0; c < grid; ++c) std::printf("%d %d\n", c, (int)v[c]);
+        } else if (!std::strcmp(kind, "tile")) {
+            int t, h, p, l, fits, sms;
+            if (std::scanf("%d %d %d %d %d %d", &t, &h, &p, &l, &fits, &sms) != 6) return 2;
+            std::printf("tile %d\n", kvx::simt_tile_tokens(t, h, p, l, fits != 0, sms));
         } else {
             return 2;
         }

@@ -10,7 +10,9 @@ helpers compute:
 - rope_schedule_ok: the rotary-width rule (0, or a multiple of 16 in [16, head_dim]);
 - pair_v_shares (`kvx_schedule.h`): the identity-alignment kernel's V shares form a permutation
   of the CTAs, and under the split's own cost model the costliest CTA costs no more than with
-  each CTA taking the mirrored V share.
+  each CTA taking the mirrored V share;
+- simt_tile_tokens: the CUDA-core kernel's 32-token tiles begin at two CTAs for each SM of the
+  device, whatever their number.
 """
 import os
 import shutil
@@ -110,3 +112,13 @@ def test_v_shares_are_a_permutation_that_lowers_the_costliest_cta(probe, grid, u
     paired = max(k[c] + vc[v[c]] for c in range(grid))
     mirrored = max(k[c] + vc[grid - 1 - c] for c in range(grid))
     assert paired <= mirrored + 1e-9
+
+
+@pytest.mark.parametrize("sms", [1, 76, 132, 152, 160])
+def test_cuda_core_tiles_follow_the_device(probe, sms):
+    """One head, one CTA a tile, one layer: 2 CTAs (K and V) for every 32 tokens."""
+    at = 32 * (sms - 1) + 1       # the first token count with sms tiles, so 2 sms CTAs
+    lines = [f"tile {t} 1 1 1 {fits} {sms}" for t, fits in ((at - 1, 1), (at, 1), (at, 0), (32 * 4096, 1))]
+    if at == 1:
+        lines = lines[1:]
+    assert probe(lines) == ["tile 16", "tile 32", "tile 16", "tile 32"][4 - len(lines):]
