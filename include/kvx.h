@@ -294,8 +294,9 @@ typedef struct {
     int32_t path;               /* KVX_PATH_SIMT or KVX_PATH_TCGEN05 */
     int32_t group_in;           /* in: input width of one translator matrix */
     int32_t n_tile;             /* output columns per tensor-core tile (tcgen05) */
-    int32_t smem_bytes;         /* dynamic shared memory per CTA */
-    int32_t threads;            /* threads per CTA */
+    int32_t smem_bytes;         /* dynamic shared memory per CTA (CUDA-core kernel: of the larger of its two
+                                 * tiles that fits; small calls take the other) */
+    int32_t threads;            /* threads per CTA (tcgen05: of the kernel that takes calls with spans) */
     int32_t num_sms;            /* SMs of the device */
     int64_t weight_bytes;       /* device bytes held for weights */
     int64_t table_bytes;        /* device bytes held for RoPE tables */

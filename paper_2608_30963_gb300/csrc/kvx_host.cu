@@ -641,7 +641,7 @@ extern "C" KVX_API kvx_status kvx_get_info(const kvx_translator* tr, kvx_transla
     info->n_tile = tr->path == KVX_PATH_TCGEN05 ? tr->tc.n_tile : 0;
     info->smem_bytes = tr->path == KVX_PATH_TCGEN05 ? tr->tc.smem_bytes
                                                     : (int)simt_smem_bytes(tr->in_dim, tr->desc.dst.head_dim);
-    info->threads = tr->path == KVX_PATH_TCGEN05 ? tr->tc.threads : 256;
+    info->threads = tr->path != KVX_PATH_TCGEN05 ? kSimtThreads : tr->row_plan ? kRowsThreads : tr->tc.threads;
     info->num_sms = tr->num_sms;
     info->weight_bytes = (int64_t)tr->w_bytes;
     info->table_bytes = (int64_t)tr->rope_bytes;

@@ -24,7 +24,7 @@ struct TcConfig {
     int n_tile;        // output columns per MMA tile
     int n_split;       // d_t / n_tile
     int smem_bytes;
-    int threads;
+    int threads;       // of the window kernel
     int ok;            // geometry supported
     int hpu;           // target heads of one unit of the window kernel
 };
@@ -47,6 +47,7 @@ cudaError_t launch_translate_tc(const TranslateParams& P, const TcConfig& cfg, i
 
 // spans over gathered source rows (kvx_tc_rows.cu): one head per unit, inputs of up to 256 channels or a
 // multiple of 256, whole-head rotations.  Same chunks and launches as launch_translate_tc; it also leaves the window plan.
+constexpr int kRowsThreads = 640;   // threads of a CTA
 bool rows_supported(int in_dim, int dt, int ds, int share);
 // one head's rows lie within 2^32 16-byte units, as the plan's row offsets count them
 bool rows_offsets_fit(const TranslateParams& P);

@@ -84,6 +84,9 @@ __global__ void tc_weight_relayout_kernel(const __nv_bfloat16* __restrict__ wk, 
     *reinterpret_cast<uint4*>(img + off) = make_uint4(v[0], v[1], v[2], v[3]);
 }
 
+// the B-loader warp (the last one) only when the weights stream
+int tc_threads(const TcLaunch& L) { return L.n_b > 1 ? kThreads : kThreads - 32; }
+
 }  // namespace
 
 TcConfig tc_config(int in_dim, int dt, int ds, int share)
@@ -94,6 +97,7 @@ TcConfig tc_config(int in_dim, int dt, int ds, int share)
     c.n_tile = L.n_tile;
     c.n_split = L.n_split;
     c.smem_bytes = kSmemMax;
+    c.threads = tc_threads(L);
     c.hpu = L.hpu;
     c.ok = 1;
     return c;
@@ -119,9 +123,7 @@ static cudaError_t launch_span_ds(int grid, cudaStream_t stream, const Translate
 {
     const cudaError_t e = smem_opt_in<translate_tc_kernel<DS, MULTI>>(kSmemMax);
     if (e != cudaSuccess) return e;
-    // the B-loader warp (the last one) only when the weights stream
-    const int threads = L.n_b > 1 ? kThreads : kThreads - 32;
-    return launch_pdl(translate_tc_kernel<DS, MULTI>, grid, threads, kSmemMax, stream, P, L);
+    return launch_pdl(translate_tc_kernel<DS, MULTI>, grid, tc_threads(L), kSmemMax, stream, P, L);
 }
 template <int DS>
 static cudaError_t launch_span(int grid, cudaStream_t stream, const TranslateParams& P, const TcLaunch& L)

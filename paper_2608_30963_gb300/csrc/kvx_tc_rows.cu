@@ -61,6 +61,7 @@ constexpr int kEpiParts = kNumEpiWarps / 4;   // epilogue warps per TMEM lane qu
 constexpr int kXfWarp0 = kEpiWarp0 + kNumEpiWarps;
 constexpr int kNumXfWarps = 8;
 constexpr int kThreads = (kXfWarp0 + kNumXfWarps) * 32;
+static_assert(kThreads == kRowsThreads, "reported by kvx_get_info");
 
 constexpr int kMaxB = 8;                            // weight ring slots (streamed)
 constexpr int kBarBFull = 0, kBarBEmpty = kMaxB;    // +weight slot

@@ -659,3 +659,22 @@ def test_span_kernels_agree_on_either_side_of_the_dense_rule(Hs, ds, Ht, dt, law
     assert not a.isnan().any() and not b.isnan().any()
     for kv in range(2):
         assert (a[kv] - b[kv]).norm() <= 2.0 ** -8 * 1.5 * b[kv].norm(), (kv, (a[kv] - b[kv]).norm() / b[kv].norm())
+
+
+@pytest.mark.parametrize("kw,path,threads", [
+    (dict(path=kvx.KVX_PATH_SIMT), kvx.KVX_PATH_SIMT, 128),
+    (dict(), kvx.KVX_PATH_TCGEN05, 640),                                       # row gather: 20 warps
+    (dict(form=kvx.KVX_FORM_DENSE), kvx.KVX_PATH_TCGEN05, 608),                # windows, weights streamed: 19 warps
+    (dict(rotary_dim=64), kvx.KVX_PATH_TCGEN05, 576),                          # windows, weights resident: 18 warps
+], ids=["simt", "rows", "windows_streamed", "windows_resident"])
+def test_info_reports_the_kernel_that_runs(kw, path, threads):
+    kw = dict(kw)
+    rd = kw.pop("rotary_dim", 0)
+    n_in = 4 * 128 if "form" in kw else 2 * 128
+    w = torch.zeros((2, 2, n_in, 128), dtype=torch.bfloat16, device="cuda")
+    tr = kvx.Translator(synth.ModelGeom(2, 4, 128, 1e4, rotary_dim=rd), synth.ModelGeom(2, 2, 128, 1e4, rotary_dim=rd), w, w,
+                        layer_map=[0, 1], **kw)
+    info = tr.info()
+    assert (info.path, info.threads, info.num_sms) == (path, threads, torch.cuda.get_device_properties(0).multi_processor_count)
+    # 32 tokens of 256 + 4 floats and two blocks of 8 rows of W by 128 channels
+    assert info.smem_bytes == (32 * (n_in + 4) * 4 + 2 * 8 * 128 * 4 if path == kvx.KVX_PATH_SIMT else 227 * 1024)
