@@ -187,3 +187,27 @@ def test_static_entry_rejects_bad_descriptions_without_touching_cuda(lib, src, d
     assert words in lib.kvx_static_last_error().decode()
     assert lib.kvx_translate_static(None, p, p, ctypes.byref(s), ctypes.byref(t), ctypes.byref(o), None, None) == \
         kvx.KVX_ERR_INVALID_ARG
+
+
+def test_cache_pointers_are_those_the_objects_report():
+    """Tensors, layers without a cache, a tensor subclass with a data_ptr of its own and objects
+    that are no tensors."""
+    torch = pytest.importorskip("torch")
+
+    class Shifted(torch.Tensor):
+        def data_ptr(self):
+            return super().data_ptr() + 16
+
+    class Other:
+        def data_ptr(self):
+            return 2 ** 63 + 32
+
+    t = [torch.zeros(4) for _ in range(3)]
+    s = [torch.zeros(4).as_subclass(Shifted) for _ in range(2)]
+    base = [torch.Tensor.data_ptr(x) for x in s]
+    p = [x.data_ptr() for x in t]
+    for objs, want in ((t, p), ([t[0], None, t[2]], [p[0], None, p[2]]), ([None, t[1]], [None, p[1]]), ([], []),
+                       (s, [b + 16 for b in base]), ([Other(), t[0]], [2 ** 63 + 32, p[0]]),
+                       ([t[0], Other()], [p[0], 2 ** 63 + 32]), ([torch.nn.Parameter(t[0])], [p[0]]), (tuple(t), p)):
+        got = kvx._ptr_array(objs)
+        assert [got[i] for i in range(len(objs))] == want
