@@ -112,7 +112,7 @@ struct TranslateParams {
                         // unit (destinations on another device, reached over the peer mapping)
     // diagnostics of the bounded waits (kvx_debug_stall_next_translate): 0 = off
     unsigned long long wait_ns;   // bound of each on-chip wait instead of ~1 s
-    int stall_unit1;              // identity kernel: CTA 0's producer issues no copies from its
+    int stall_unit1;              // identity and row-gather kernels: CTA 0's copying warps issue none from its
                                   // (stall_unit1 - 1)-th unit on, so the waits for them run out
     unsigned* status;
     // weights (layout depends on the kernel)

@@ -32,12 +32,12 @@
 // Dense spans.  Further rows that the side buffer has no room for are read from memory by the prologue, with their
 // latency exposed; a window (kvx_tc_window.cuh) holds 48 rows of a 32-token sub-tile and is copied ahead.  The spans
 // are known on the device only.  Where the source may hold 1.5 rows or more for each target token the kernel is
-// launched in a form (DENSE) that counts, over the plan's tiles, the further rows beyond the side buffer (o), the
+// launched in a form (kDense) that counts, over the plan's tiles, the further rows beyond the side buffer (o), the
 // tokens of several rows (m) and the rows of the tokens outside their windows (w), and runs the window kernel's body
 // where o + 2 m - w / 4 exceeds dense_sum a tile (rows_layout).  With fewer source rows the spans can only be dense
 // where they overlap, and the plain form runs: the count and the second body cost it up to 2% (70B -> 7B shapes, 8192
-// tokens: 513 us against 503; 1.5B -> Gemma-2B shapes, a ragged batch of 1574: 98.8 against 98.0).  4096 tokens, 8 layers of 128 x 128 heads grouped by two, us here and in windows:
-// spans of 1.3 rows 59 and 79, of 1.6 86 and 94, of 2 119 and 114, of two each 112 and 91, of 8 to 16 964 and 803.
+// tokens: 513 us against 503; 1.5B -> Gemma-2B shapes, a ragged batch of 1574: 98.8 against 98.0).  4096
+// tokens, 8 layers of 128 x 128 heads grouped by two, us here and in windows: spans of 1.3 rows 59 and 79, of 1.6 86 and 94, of 2 119 and 114, of two each 112 and 91, of 8 to 16 964 and 803.
 #include "kvx_common.cuh"
 #include "kvx_kernels.h"
 #include "kvx_span_plan.cuh"
@@ -274,13 +274,15 @@ __device__ __forceinline__ uint4 pack8(const float (&a)[8], float f)
                       pack_bf16(a[6] * f, a[7] * f));
 }
 // HS: half head_dim of the source (32, 64 or 128); HEADS: source heads of a K group; STREAM: several K groups,
-// weights streamed (else a resident image); DENSE: the spans may be dense (see the top), D is the window kernel's
-// launch over the same tokens
-template <int HS, int HEADS, bool STREAM, bool DENSE>
+// weights streamed (else a resident image).  MODE: kDense, the spans may be dense (see the top), D is the window
+// kernel's launch over the same tokens; kDiag, the diagnostics of the bounded waits.
+constexpr int kPlain = 0, kDense = 1, kDiag = 2;
+template <int HS, int HEADS, bool STREAM, int MODE>
 __global__ void __launch_bounds__(kThreads, 1)
 translate_rows_kernel(const __grid_constant__ TranslateParams P, const __grid_constant__ RowsLaunch L,
                       const __grid_constant__ window::TcLaunch D)
 {
+    constexpr bool DENSE = MODE == kDense;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
     uint8_t* sB = smem + L.off_b;
@@ -675,6 +677,7 @@ translate_rows_kernel(const __grid_constant__ TranslateParams P, const __grid_co
         for (; x.more() && ok; x.next()) {
             cur[0] = nxt[0];
             cur[1] = nxt[1];
+            if (MODE == kDiag && blockIdx.x == 0 && x.it + 1 == P.stall_unit1) break;
             // the prologue's copy of the tile's row entries
             if (!W.wait(bar(kBarEntEmpty + ent_cnt % kEntTabs), ((ent_cnt / kEntTabs) & 1) ^ 1)) break;
 #pragma unroll
@@ -889,23 +892,30 @@ bool rows_layout(int in_dim, int dt, int ds, int share, RowsLaunch& L)
     return cols <= 512;
 }
 
-template <int HS, int HEADS, bool STREAM, bool DENSE>
+template <int HS, int HEADS, bool STREAM, int MODE>
 cudaError_t launch_rows_v(int grid, cudaStream_t stream, const TranslateParams& P, const RowsLaunch& L,
                           const window::TcLaunch& D)
 {
-    const cudaError_t e = smem_opt_in<translate_rows_kernel<HS, HEADS, STREAM, DENSE>>(kSmemMax);
+    const cudaError_t e = smem_opt_in<translate_rows_kernel<HS, HEADS, STREAM, MODE>>(kSmemMax);
     if (e != cudaSuccess) return e;
-    return launch_pdl(translate_rows_kernel<HS, HEADS, STREAM, DENSE>, grid, kThreads, kSmemMax, stream, P, L, D);
+    return launch_pdl(translate_rows_kernel<HS, HEADS, STREAM, MODE>, grid, kThreads, kSmemMax, stream, P, L, D);
+}
+template <int HS, int HEADS, bool STREAM>
+cudaError_t launch_rows_s(int grid, int mode, cudaStream_t stream, const TranslateParams& P, const RowsLaunch& L,
+                          const window::TcLaunch& D)
+{
+    // (one shape is compiled for the diagnostics, to save the others' compile time)
+    if constexpr (HS == 64 && HEADS == 2)
+        if (mode == kDiag) return launch_rows_v<HS, HEADS, STREAM, kDiag>(grid, stream, P, L, D);
+    return mode == kDense ? launch_rows_v<HS, HEADS, STREAM, kDense>(grid, stream, P, L, D)
+                          : launch_rows_v<HS, HEADS, STREAM, kPlain>(grid, stream, P, L, D);
 }
 template <int HS, int HEADS>
-cudaError_t launch_rows(int grid, bool dense, cudaStream_t stream, const TranslateParams& P, const RowsLaunch& L,
+cudaError_t launch_rows(int grid, int mode, cudaStream_t stream, const TranslateParams& P, const RowsLaunch& L,
                         const window::TcLaunch& D)
 {
-    if (L.kgs > 1)
-        return dense ? launch_rows_v<HS, HEADS, true, true>(grid, stream, P, L, D)
-                     : launch_rows_v<HS, HEADS, true, false>(grid, stream, P, L, D);
-    return dense ? launch_rows_v<HS, HEADS, false, true>(grid, stream, P, L, D)
-                 : launch_rows_v<HS, HEADS, false, false>(grid, stream, P, L, D);
+    return L.kgs > 1 ? launch_rows_s<HS, HEADS, true>(grid, mode, stream, P, L, D)
+                     : launch_rows_s<HS, HEADS, false>(grid, mode, stream, P, L, D);
 }
 
 }  // namespace
@@ -947,6 +957,7 @@ cudaError_t launch_translate_rows(const TranslateParams& P, int num_sms, void* w
     L.rows = rows;
     // the source may hold 1.5 rows or more for each target token (what the host knows: the caches' capacity)
     const bool dense = P.span_lo && 2ll * P.batch * P.src_max_seq >= 3ll * P.T_total;
+    const int mode = P.wait_ns != 0 || P.stall_unit1 != 0 ? kDiag : dense ? kDense : kPlain;
     L.share = share > 1 && P.Ht % share == 0 ? share : 1;
     for (int t0 = 0; t0 < P.T_total; t0 += chunk) {
         const int t1 = P.T_total - t0 < chunk ? P.T_total : t0 + chunk;
@@ -959,12 +970,12 @@ cudaError_t launch_translate_rows(const TranslateParams& P, int num_sms, void* w
         if (e != cudaSuccess) return e;
         ++*launches;
         switch (P.ds * 8 + L.nblk * kBlockK / P.ds) {   // source heads of a K group
-        case 64 * 8 + 1: e = launch_rows<32, 1>(grid, dense, stream, P, L, D); break;
-        case 64 * 8 + 2: e = launch_rows<32, 2>(grid, dense, stream, P, L, D); break;
-        case 64 * 8 + 4: e = launch_rows<32, 4>(grid, dense, stream, P, L, D); break;
-        case 128 * 8 + 1: e = launch_rows<64, 1>(grid, dense, stream, P, L, D); break;
-        case 128 * 8 + 2: e = launch_rows<64, 2>(grid, dense, stream, P, L, D); break;
-        case 256 * 8 + 1: e = launch_rows<128, 1>(grid, dense, stream, P, L, D); break;
+        case 64 * 8 + 1: e = launch_rows<32, 1>(grid, mode, stream, P, L, D); break;
+        case 64 * 8 + 2: e = launch_rows<32, 2>(grid, mode, stream, P, L, D); break;
+        case 64 * 8 + 4: e = launch_rows<32, 4>(grid, mode, stream, P, L, D); break;
+        case 128 * 8 + 1: e = launch_rows<64, 1>(grid, mode, stream, P, L, D); break;
+        case 128 * 8 + 2: e = launch_rows<64, 2>(grid, mode, stream, P, L, D); break;
+        case 256 * 8 + 1: e = launch_rows<128, 1>(grid, mode, stream, P, L, D); break;
         default: return cudaErrorNotSupported;
         }
         if (e != cudaSuccess) return e;
