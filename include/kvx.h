@@ -225,7 +225,7 @@ typedef struct {
  * rows of distinct target tokens are written exactly once.
  * Calls on one translator must be ordered: issue them on one stream, or serialise them on the
  * host and order them on the device (events).  The translator owns per-call state that two
- * overlapping calls would share: the span kernel's plan buffer on the device, the cache of
+ * overlapping calls would share: the span kernels' plan buffers on the device, the cache of
  * source tensor descriptors and the launch count on the host.  Distinct translators may run
  * concurrently on different streams and host threads. */
 KVX_API kvx_status kvx_translate(kvx_translator* tr, const kvx_src_kv* src, const kvx_tgt_tokens* tgt,
@@ -306,7 +306,7 @@ KVX_API kvx_status kvx_get_info(const kvx_translator* tr, kvx_translator_info* i
 
 /* Kernel launches the most recent kvx_translate call on this translator made (for
  * launch accounting): 1 for the identity-alignment and CUDA-core kernels; 2 per
- * chunk of up to 65536 target tokens for the span kernel (a span-plan launch and the
+ * chunk of up to 65536 target tokens for the span kernels (a span-plan launch and the
  * translation launch).  0 before the first call and after a call with no tokens. */
 KVX_API int32_t kvx_launches_per_translate(const kvx_translator* tr);
 

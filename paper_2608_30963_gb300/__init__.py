@@ -426,7 +426,7 @@ class Translator:
         _check(lib().kvx_debug_stall_next_translate(VP(self.handle), unit, wait_us))
 
     def span_plan_stats(self, stream=None) -> dict:
-        """Token-span plan of the last translate (span kernel only): sub-tiles, tokens staged in
+        """Token-span windows of the last translate (calls with spans only): sub-tiles, tokens staged in
         their sub-tile's window, tokens gathered from global memory."""
         return kvx_span_plan_stats(self.handle, _stream(stream))
 

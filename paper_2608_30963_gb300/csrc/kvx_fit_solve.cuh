@@ -16,7 +16,7 @@
 // instruction fetch was most of the factor's time.
 // Measured, factor and solves: 112 systems of 256 x 128 in fp32 151 and 122 us (2.0 ms with an unblocked
 // factor and one thread per right-hand side); 208 systems of 128 x 256 in pairs 220 and 464 us, the
-// latter near the fp32 pipe's rate.
+// latter near the fp32 pipe's rate (its scaling included).
 //
 // Arithmetic is a parameter.  F32: fp32, for systems the pivots show to be well conditioned.  Pair:
 // unevaluated sums h + l of two floats (about 48 bits), products exact by FMA (Dekker's two-product) and
@@ -28,8 +28,8 @@
 // Cholesky solve's rounding errors do not depend on it, but the low words of a pair keep their bits only above 2^-102,
 // so without it systems of small sums (channels of 1e-16 and below) would fall back to fp32.  It also makes the
 // pivots show what the pairs have to resolve: channel scales do not count, nearly dependent channels do.
-// Where the scaled pivots show a condition number above 4096 (max_cond) 48 bits no longer leave W's error to the
-// rounding of its elements, and the system goes to the double kernel.
+// Systems whose scaled pivots show a condition number above max_cond go to the double kernel: 48 bits begin to show
+// in W there.
 #pragma once
 
 #include <climits>

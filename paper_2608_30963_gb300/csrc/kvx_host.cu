@@ -33,13 +33,13 @@ struct kvx_translator {
     int rope_same = 0;           // source and target turns identical (same d, same frequencies)
     unsigned* status = nullptr;
     TcConfig tc{};
-    // span plan of the tensor-core span kernel: sub-tile windows and per-token entries
+    // window plan of the tensor-core span kernels: sub-tile windows and per-token entries
     // for up to kPlanTokens target tokens per launch (longer calls run in chunks)
     static constexpr int kPlanTokens = 1 << 16;
     void* plan = nullptr;
-    void* row_plan = nullptr;    // row plan of the row-gather span kernel, where the geometry takes it
+    void* row_plan = nullptr;    // row plan of the row-gather kernel, where the geometry takes it
     int last_launches = 0;       // kernel launches of the most recent kvx_translate
-    int last_span_tokens = 0;    // target tokens of the most recent call if it ran the span kernel, else 0
+    int last_span_tokens = 0;    // target tokens of the most recent call if it ran a span kernel, else 0
     int dbg_stall_unit1 = 0;     // kvx_debug_stall_next_translate, for the next call only
     unsigned long long dbg_wait_ns = 0;
     // encoded source tensor maps of the identity-alignment kernel, a few per (target layer, K|V)
@@ -472,7 +472,7 @@ static kvx_status translate_impl(kvx_translator* tr, const kvx_src_kv* src, cons
     if (tgt->total_tokens == 0) return KVX_OK;
     P.plain_stores = plain_stores;
     cudaError_t ce;
-    // partial rotary heads (rotary_dim < head_dim on either side) take the span kernel, which
+    // partial rotary heads (rotary_dim < head_dim on either side) take the window kernel, which
     // pairs channels at rotary_dim/2; the identity kernel pairs whole heads
     const bool whole_head_rope = rope_rot_dim(D.src) == D.src.head_dim && rope_rot_dim(D.dst) == D.dst.head_dim;
     if (tr->path == KVX_PATH_TCGEN05 && !tgt->span_lo && whole_head_rope &&
@@ -663,7 +663,7 @@ extern "C" KVX_API kvx_status kvx_span_plan_stats(kvx_translator* tr, void* stre
 {
     if (!tr || !counts) return fail(KVX_ERR_INVALID_ARG, "span_plan_stats: NULL argument");
     if (tr->last_span_tokens <= 0 || !tr->plan)
-        return fail(KVX_ERR_INVALID_ARG, "span_plan_stats: the last kvx_translate did not run the span kernel");
+        return fail(KVX_ERR_INVALID_ARG, "span_plan_stats: the last kvx_translate did not run a span kernel");
     int nsub = 0, ent_off = 0;
     tc_plan_layout(tr->last_span_tokens, kvx_translator::kPlanTokens, &nsub, &ent_off);
     std::vector<int4> ent((size_t)nsub * 32);

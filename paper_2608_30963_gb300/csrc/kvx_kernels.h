@@ -29,14 +29,14 @@ struct TcConfig {
     int hpu;           // target heads of one unit of the window kernel
 };
 // share: target heads that read the same input rows (share_heads); it decides how many heads
-// one unit of the span kernel covers and so the weight images' output split n_tile.
+// one unit of the window kernel covers and so the weight images' output split n_tile.
 TcConfig tc_config(int in_dim, int dt, int ds, int share);
 size_t tc_weight_image_bytes(int in_dim, int dt, int Lt, int Ht);
 // rhalf_t: rotating pairs of the target head (rotary_dim/2; d_t/2 unless partial rotary)
 cudaError_t launch_tc_weight_relayout(const void* w_k, const void* w_v, void* image, int Lt, int Ht, int in_dim,
                                       int dt, int n_tile, int rhalf_t, cudaStream_t stream);
 size_t tc_plan_bytes(int tokens);
-// Where the plan of the last chunk of a span-kernel call lives in the plan buffer: its
+// Where the window plan of the last chunk of a call with spans lives in the plan buffer: its
 // sub-tile headers start at int4 0, its per-token entries (32 per sub-tile) at int4
 // *ent_off; *nsub sub-tiles.  T_total: target tokens of the call.
 void tc_plan_layout(int T_total, int plan_tokens, int* nsub, int* ent_off);
@@ -46,7 +46,7 @@ cudaError_t launch_translate_tc(const TranslateParams& P, const TcConfig& cfg, i
                                 int plan_tokens, cudaStream_t stream, int* launches);
 
 // spans over gathered source rows (kvx_tc_rows.cu): one head per unit, inputs of up to 256 channels or a
-// multiple of 256, whole-head rotations.  Same chunks and launches as launch_translate_tc; it also leaves the window plan.
+// multiple of 256, whole-head rotations (dense spans in the window kernel's body).  Same chunks and launches as launch_translate_tc; it also leaves the window plan.
 constexpr int kRowsThreads = 640;   // threads of a CTA
 bool rows_supported(int in_dim, int dt, int ds, int share);
 // one head's rows lie within 2^32 16-byte units, as the plan's row offsets count them

@@ -11,7 +11,7 @@
 // It serves the float32 caches and any geometry the tensor-core kernel does not take.  Paper:
 // Section 5 (T_theta per layer and KV head).
 //
-// Bound: fp32 FMA issue (128 a clock and SM).  Each output is one accumulator in ascending input
+// Bound: shared-memory reads of W and A (70% of that pipe) and fp32 FMA issue (48% of the slots).  Each output is one accumulator in ascending input
 // order.  1000 tokens of 7B -> 1.5B shapes (3.7 G FMA): 199 us; 608 us with a thread per output channel
 // and scalar reads of A and W.
 #include "kvx_common.cuh"

@@ -77,7 +77,7 @@ __device__ __forceinline__ void resolve_dst(const TranslateParams& P, const SeqV
 }
 
 // Window plan of one 32-token sub-tile, read by every (layer, head, K|V) group of the window kernel
-// (kvx_tc.cu) and counted by kvx_span_plan_stats:
+// (kvx_tc_window.cuh) and counted by kvx_span_plan_stats:
 //   header  {b0, c0, rows, 0}: the window of source rows [c0, c0 + rows) of sequence b0
 //   entries {w0, lo, hi, b} x 32, longest span first: w0 = window row of the span
 //           start (low 16 bits, signed; -1: read from global memory) | A row within

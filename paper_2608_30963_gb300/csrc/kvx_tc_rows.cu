@@ -5,7 +5,7 @@
 // a token of one source row (three in four) is in place when its copies land: for V nothing is left to
 // do, for K the row is un-rotated where it lies.  Only tokens with more rows are averaged in registers,
 // from A and from a side buffer that a warp of its own fills with the tile's further rows.  Building every
-// row in registers from a staged window of source rows (kvx_tc.cu) leaves the tensor core waiting for the
+// row in registers from a staged window of source rows (kvx_tc_window.cuh) leaves the tensor core waiting for the
 // chain of eight-lane steps that do it.
 //
 // Row plan (span_rows_kernel, once per translation, read by every (layer, head, K|V) group): per tile

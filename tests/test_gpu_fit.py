@@ -272,9 +272,9 @@ def test_fit_fp32_tiny_matches_oracle_tightly():
 def test_fit_ill_conditioned_calibration_matches_oracle():
     """A calibration set whose two source heads nearly coincide (head 1 = head 0 + 3e-3 noise):
     X^T X + lambda I has a condition number above 1e6, where an fp32 Cholesky factor loses most
-    of its digits.  The fitter sees it in the factor's pivots and solves those systems again in
-    pairs of floats (status bit 0x40); W then matches the oracle's fp64 solution within the bound of
-    the fp32 sums and a double factorisation.  fp32 caches, so the rows carry no bf16 rounding."""
+    of its digits.  The fitter sees it in the factor's pivots and solves those systems again, in
+    pairs of floats or double (status bit 0x40); W then matches the oracle's fp64 solution within the
+    bound of the fp32 sums and a double factorisation.  fp32 caches, so the rows carry no bf16 rounding."""
     spec = SPECS["tiny_fp32"]
     c = make_case(spec, [456])
     rng = np.random.default_rng(21)
@@ -287,7 +287,7 @@ def test_fit_ill_conditioned_calibration_matches_oracle():
     tv = tv + np.float32(1e-3) * rng.standard_normal(tv.shape).astype(np.float32)
     lam = 1e-4
     gk, gv, bits, _ = _fit_gpu(c, tk, tv, lam)
-    assert bits & 0x40, f"status 0x{bits:x}: no system was solved in double"
+    assert bits & 0x40, f"status 0x{bits:x}: no system was solved again"
     assert not bits & 0x20
     ok, ov = oracle_problem(c).fit(list(tk), list(tv), lam)
     p = oracle_problem(c)

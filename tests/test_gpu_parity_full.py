@@ -8,9 +8,11 @@
   aligned on the device by kvx_build_alignment and fed to kvx_translate: a finer target
   (several target tokens on one source token), a coarser one (long spans), equal grains, and
   single-byte source tokens under 6-byte target tokens, whose 32-token sub-tiles need more
-  source rows than the span kernel's 48-row window holds, so the global-memory gather runs on
+  source rows than the window kernel's 48-row window holds, so that its global-memory gather runs on
   every full sub-tile (checked through the plan diagnostics against the plan rule).
 - Non-monotone and overlapping spans, which no tokenizer pair gives but the interface allows.
+Whole-head rotations run in the row-gather kernel (its own walk or, dense spans, the window kernel's body),
+partial rotary heads in the window kernel.
 """
 import dataclasses
 
@@ -28,7 +30,7 @@ from harness import compare, explicit_span_workload, make_case, oracle_problem, 
 pytestmark = pytest.mark.gpu
 SPECS = synth.config_specs()
 PATHS = [kvx.KVX_PATH_SIMT, kvx.KVX_PATH_AUTO]
-WINDOW_CAP = 48   # source rows one sub-tile window of the span kernel stages
+WINDOW_CAP = 48   # source rows one sub-tile window of the window kernel stages
 
 
 @pytest.fixture(scope="module", autouse=True)
@@ -97,7 +99,13 @@ def _expected_plan(wl, cap=WINDOW_CAP):
 
 MIXES = {"target_finer_5_2": (5.0, 2.0), "target_coarser_2_6": (2.0, 6.0), "equal_1_1": (1.0, 1.0),
          "byte_source_1_6": (1.0, 6.0)}
-GEOMS = {"gemma_expansion": ("qwen1p5b_to_gemma2b_1k", 3, 2), "llama_grouped": ("llama70b_to_qwen7b_8k", 3, 2)}
+GEOMS = {"gemma_expansion": ("qwen1p5b_to_gemma2b_1k", 3, 2), "llama_grouped": ("llama70b_to_qwen7b_8k", 3, 2),
+         "llama_partial_rotary": ("llama70b_to_qwen7b_8k", 3, 2)}
+
+
+def _partial_rotary(spec):
+    return dataclasses.replace(spec, src=dataclasses.replace(spec.src, rotary_dim=64),
+                               dst=dataclasses.replace(spec.dst, rotary_dim=64))
 
 
 @pytest.mark.parametrize("path", PATHS, ids=["simt", "auto"])
@@ -107,6 +115,8 @@ def test_spans_from_independent_tokenizations(mix, geom, path):
     from gpu_harness import DeviceCase, i32
     base, Ls, Lt = GEOMS[geom]
     spec = _shrink(SPECS[base], Ls, Lt)
+    if geom == "llama_partial_rotary":
+        spec = _partial_rotary(spec)
     ms, mt = MIXES[mix]
     wl = tokenization_workload(spec, [2600, 37, 1, 900], ms, mt, key=7 + list(MIXES).index(mix))
     c = make_case(spec, wl=wl)
@@ -141,10 +151,13 @@ def test_spans_from_independent_tokenizations(mix, geom, path):
 
 
 @pytest.mark.parametrize("path", PATHS, ids=["simt", "auto"])
+@pytest.mark.parametrize("rotary", ["whole", "partial"])
 @pytest.mark.parametrize("kind", ["reversed", "random_overlapping"])
-def test_non_monotone_spans(kind, path):
+def test_non_monotone_spans(kind, rotary, path):
     from gpu_harness import DeviceCase
     spec = _shrink(SPECS["llama70b_to_qwen7b_8k"], 3, 2)
+    if rotary == "partial":
+        spec = _partial_rotary(spec)
     r = np.random.default_rng(41)
     src_lens, los, his = [], [], []
     for b, T in enumerate([700, 130]):
