@@ -661,9 +661,10 @@ EncodeTiled encoder()
 
 bool aligned_supported(int in_dim, int dt, int ds, int share, int Lt, int batch, int kl)
 {
-    // one source layer per target layer (one tensor map each) and a resident B image
+    // one source layer per target layer (one tensor map each) and a resident B image (the window kernel, which
+    // streams it for units of several heads, may have left it whole: 256 channels onto 256)
     TcConfig c = tc_config(in_dim, dt, ds, share);
-    return c.ok && in_dim <= 256 && kl == 1 && Lt <= KVX_MAX_ALIGNED_LAYERS && batch <= KVX_MAX_ALIGNED_BATCH &&
+    return c.ok && in_dim <= 256 && in_dim * c.n_tile <= 32768 && kl == 1 && Lt <= KVX_MAX_ALIGNED_LAYERS && batch <= KVX_MAX_ALIGNED_BATCH &&
            encoder() != nullptr;
 }
 

@@ -678,3 +678,28 @@ def test_info_reports_the_kernel_that_runs(kw, path, threads):
     assert (info.path, info.threads, info.num_sms) == (path, threads, torch.cuda.get_device_properties(0).multi_processor_count)
     # 32 tokens of 256 + 4 floats and two blocks of 8 rows of W by 128 channels
     assert info.smem_bytes == (32 * (n_in + 4) * 4 + 2 * 8 * 128 * 4 if path == kvx.KVX_PATH_SIMT else 227 * 1024)
+
+
+@pytest.mark.parametrize("Hs,ds,Ht,dt", [(4, 64, 2, 256), (4, 64, 4, 256), (2, 64, 2, 256), (2, 128, 2, 128), (2, 64, 4, 128)])
+def test_dense_form_with_one_tokenizer(Hs, ds, Ht, dt):
+    """The dense form without span arrays: weight images that the identity kernel keeps resident, and 256 channels onto
+    256, which it cannot (128 KB).  Against the CUDA-core kernel, as above."""
+    L, T = 2, 300
+    i32 = lambda x: torch.tensor(np.asarray(x), dtype=torch.int32, device="cuda")
+    gen = torch.Generator(device="cuda").manual_seed(12)
+    rnd = lambda *sh: torch.randn(sh, device="cuda", generator=gen).to(torch.bfloat16)
+    src = [[rnd(1, Hs, T, ds) for _ in range(L)] for _ in range(2)]
+    w = [rnd(L, Ht, Hs * ds, dt) for _ in range(2)]
+    outs = []
+    for path in (kvx.KVX_PATH_TCGEN05, kvx.KVX_PATH_SIMT):
+        tr = kvx.Translator(synth.ModelGeom(L, Hs, ds, 1e4), synth.ModelGeom(L, Ht, dt, 1e6), w[0], w[1],
+                            layer_map=list(range(L)), path=path, form=kvx.KVX_FORM_DENSE)
+        dst = [[torch.full((1, Ht, T, dt), float("nan"), dtype=torch.bfloat16, device="cuda") for _ in range(L)] for _ in range(2)]
+        tr.translate(src[0], src[1], i32([T]), i32([0, T]), T, dst[0], dst[1])
+        torch.cuda.synchronize()
+        assert tr.device_status() == 0
+        outs.append(torch.stack([torch.stack(d) for d in dst]).double())
+    a, b = outs
+    assert not a.isnan().any() and not b.isnan().any()
+    for kv in range(2):
+        assert (a[kv] - b[kv]).norm() <= 2.0 ** -8 * 1.5 * b[kv].norm(), (kv, (a[kv] - b[kv]).norm() / b[kv].norm())
