@@ -24,6 +24,8 @@
 #include <stdio.h>
 #include <string.h>
 
+#include <numeric>
+
 #include "kvx_common.cuh"
 #include "kvx_fit_solve.cuh"
 #include "kvx_kernels.h"
@@ -310,7 +312,7 @@ __global__ void __launch_bounds__(256) fit_gram_simt_kernel(const T* __restrict_
 //                pairs (8 lanes per 128-channel head), each lane taking the span mean of its
 //                chunk pair; tokens whose span leaves the window read their rows from global
 //                memory.
-//                Identity alignment ("direct" blocks): 4 teams of 3 warps, one block per team.
+//                Identity alignment ("direct" blocks): 4 teams of 4 warps, one block per team.
 //                A thread gathers its (token, chunk pair) items straight into their swizzled
 //                places with 16-byte cp.async, waits for its own copies and un-rotates K in
 //                place, one (cos, sin) per pair for every source head and, when the rotations
@@ -340,6 +342,10 @@ constexpr int kGramMaxStages = 4;
 constexpr int kGramMaxRaw = 8;
 // Direct blocks (every span one source row): the prologue warps work in teams, one 64-token block each.
 constexpr int kGramTeams = 4;
+// Block b's consumption is announced on barrier b % nze, nze = lcm(stages, teams): a barrier's phases are then all awaited
+// by one team, in order.  With a barrier a stage, and three or two stages under four teams (in + d_t > 384), a team
+// came back to a stage's barrier after several of its phases and could take one for another of the same parity.
+constexpr int kGramMaxEmpty = 12;
 constexpr int kGramMaxRows = 512;   // in + dt: one 128 x 512 fp32 accumulator fills TMEM
 constexpr int kGramMaxHeads = 6;    // source head-blocks in one input row
 
@@ -356,6 +362,7 @@ struct GramLaunch {
     int nkb;               // K-blocks of 64 tokens in the call
     int units;             // groups * mbs
     int stages;            // Z^T block ring depth
+    int nze;               // barriers that announce a consumed block (kGramMaxEmpty)
     unsigned stage_bytes;  // nrows * 128
     int raw_slots;         // raw staging ring depth
     int rcap;              // source rows one window holds
@@ -480,9 +487,9 @@ __global__ void __launch_bounds__(gram_threads(DIRECT), 1) fit_gram_tc_kernel(co
     uint8_t* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
     uint8_t* sRaw = smem + L.off_raw;
     uint64_t* sBar = reinterpret_cast<uint64_t*>(smem + L.off_bar);
-    // barriers: zfull[s] (prologue warps), zempty[s] (MMA commit), rfull[r] (loader + copies),
+    // barriers: zfull[s] (prologue warps), zempty[b % nze] (MMA commit), rfull[r] (loader + copies),
     // rempty[r] (prologue warps), dfull (MMA commit), dempty (epilogue warps), done (MMA)
-    constexpr int bZFull = 0, bZEmpty = kGramMaxStages, bRFull = 2 * kGramMaxStages, bREmpty = bRFull + kGramMaxRaw;
+    constexpr int bZFull = 0, bZEmpty = kGramMaxStages, bRFull = bZEmpty + kGramMaxEmpty, bREmpty = bRFull + kGramMaxRaw;
     constexpr int bDFull = bREmpty + kGramMaxRaw, bDEmpty = bDFull + 1, bDone = bDFull + 2;
     volatile int* sAbort = reinterpret_cast<volatile int*>(sBar + bDone + 1);
     uint32_t* sTmem = reinterpret_cast<uint32_t*>(sBar + bDone + 2);
@@ -493,10 +500,8 @@ __global__ void __launch_bounds__(gram_threads(DIRECT), 1) fit_gram_tc_kernel(co
     if (threadIdx.x == 32) sRange->init(L, P.dt);
     if (threadIdx.x == 0) {
         *sAbort = 0;
-        for (int i = 0; i < L.stages; ++i) {
-            mbar_init(bar(bZFull + i), DIRECT ? kGramTeamWarps : kGramNumXf);
-            mbar_init(bar(bZEmpty + i), 1);
-        }
+        for (int i = 0; i < L.stages; ++i) mbar_init(bar(bZFull + i), DIRECT ? kGramTeamWarps : kGramNumXf);
+        for (int i = 0; i < L.nze; ++i) mbar_init(bar(bZEmpty + i), 1);
         for (int i = 0; i < L.raw_slots; ++i) {
             mbar_init(bar(bRFull + i), 1);
             mbar_init(bar(bREmpty + i), DIRECT ? kGramTeamWarps : kGramNumXf);
@@ -518,6 +523,12 @@ __global__ void __launch_bounds__(gram_threads(DIRECT), 1) fit_gram_tc_kernel(co
     tc_fence_after();
     const uint32_t tmem_base = *sTmem;
     const Waiter W{sAbort, P.status};
+    // the stage of block `it` is free: the block before it there has been consumed
+    auto stage_free = [&](uint32_t it) -> bool {
+        if (it < (uint32_t)L.stages) return true;
+        const uint32_t b = it - (uint32_t)L.stages, n = (uint32_t)L.nze;
+        return W.wait(bar(bZEmpty + b % n), (b / n) & 1);
+    };
     const GramRange R = *sRange;
     const int in = NHD * DS, dt = P.dt;
     constexpr int heads = NHD;
@@ -559,7 +570,7 @@ __global__ void __launch_bounds__(gram_threads(DIRECT), 1) fit_gram_tc_kernel(co
                               sw128_mn_desc(st + (uint32_t)(in / 64) * colblk + k * 2048, L.lbo, L.sbo),
                               gram_idesc_dev(dt), acc);
                 }
-                umma_commit(bar(bZEmpty + s));
+                umma_commit(bar(bZEmpty + it % (uint32_t)L.nze));
                 issued = true;
                 if (last) {
                     umma_commit(bar(bDFull));
@@ -713,9 +724,9 @@ __global__ void __launch_bounds__(gram_threads(DIRECT), 1) fit_gram_tc_kernel(co
             const GramUnit x = R.at(L, blk);
             const int kv = x.g & 1, jh = x.g >> 1, h = jh % P.Ht, j = jh / P.Ht;
             const int nh = min(heads, ((x.mb + 1) * 128 + DS - 1) / DS);
-            const uint32_t s = it % (uint32_t)L.stages, ph = (it / (uint32_t)L.stages) & 1;
+            const uint32_t s = it % (uint32_t)L.stages;
             const uint32_t r = it % (uint32_t)L.raw_slots, rph = (it / (uint32_t)L.raw_slots) & 1;
-            if (!W.wait(bar(bZEmpty + s), ph ^ 1)) break;
+            if (!stage_free(it)) break;
             if (!W.wait(bar(bRFull + r), rph)) break;
             uint8_t* st = smem + (size_t)s * L.stage_bytes;
             const uint32_t st32 = smem_u32(st);
@@ -831,9 +842,9 @@ __global__ void __launch_bounds__(gram_threads(DIRECT), 1) fit_gram_tc_kernel(co
             const int kv = x.g & 1, jh = x.g >> 1, h = jh % P.Ht, j = jh / P.Ht;
             // X head-blocks this row block needs: the rows [0, (mb+1)*128) of the lower triangle
             const int nh = min(heads, ((x.mb + 1) * 128 + DS - 1) / DS);
-            const uint32_t s = it % (uint32_t)L.stages, ph = (it / (uint32_t)L.stages) & 1;
+            const uint32_t s = it % (uint32_t)L.stages;
             const uint32_t r = it % (uint32_t)L.raw_slots, rph = (it / (uint32_t)L.raw_slots) & 1;
-            if (!W.wait(bar(bZEmpty + s), ph ^ 1)) break;
+            if (!stage_free(it)) break;
             if (!W.wait(bar(bRFull + r), rph)) break;
             uint8_t* st = smem + (size_t)s * L.stage_bytes;
             const GramTok* tt = tok_tab((int)r);
@@ -1122,7 +1133,7 @@ extern "C" KVX_API kvx_status kvx_fit_accumulate(kvx_fitter* f, const kvx_src_kv
         L.stage_bytes = (unsigned)L.nrows * 128;
         L.src_row = (unsigned)ds * 2;   // rows as in the caches: whole windows move in one copy
         L.tgt_row = (unsigned)dt * 2;
-        const unsigned tail = 32 * 8 + (unsigned)(ds / 2 + dt / 2) * 8 + sizeof(GramRange);   // barriers, flags, turns, range
+        const unsigned tail = 40 * 8 + (unsigned)(ds / 2 + dt / 2) * 8 + sizeof(GramRange);   // barriers, flags, turns, range
         // identity alignment: every span is one source row (or none), gathered by the prologue
         const bool direct = P.span_lo == nullptr;
         bool fits = false;
@@ -1151,6 +1162,7 @@ extern "C" KVX_API kvx_status kvx_fit_accumulate(kvx_fitter* f, const kvx_src_kv
                 fits = 1024 + L.off_bar + tail <= (unsigned)kSmemMax;
             }
         if (!fits) return fit_fail(KVX_ERR_UNSUPPORTED, "fit_accumulate: Gram blocks do not fit shared memory");
+        L.nze = direct ? std::lcm(L.stages, kGramTeams) : L.stages;   // (staged blocks: one team)
         L.lbo = kGramK * 128;   // next 64-channel column block
         L.sbo = 1024;           // next 8-token atom row
         L.G = G;

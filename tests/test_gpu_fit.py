@@ -432,6 +432,38 @@ def test_wide_systems_from_tensor_core_sums_match_a_double_solve():
             assert _rel(got, ref) <= 2.0 ** -9 + 16 * T * 2.0 ** -24, (kv, j, _rel(got, ref))
 
 
+@pytest.mark.parametrize("ds,kl,r,dt", [(64, 3, 2, 64), (128, 3, 1, 64), (128, 3, 1, 128), (256, 1, 1, 256), (128, 2, 1, 256),
+                                        (128, 1, 2, 128)])
+def test_identity_fits_with_fewer_block_stages_than_teams(ds, kl, r, dt):
+    """Inputs and targets of 448 and 512 channels leave room for three 64-token blocks on chip, under four teams that
+    build them (384 channels: four blocks).  K un-rotated and V copied, so that teams run apart; rows of many blocks;
+    three fits.  V, whose bf16 rows are exact inputs, against numpy in double (W's rounding to bf16, 2^-9 an element, and
+    the fp32 sums' as above); K alike from fit to fit, to those two roundings."""
+    n_in, L = kl * r * ds, 5
+    T = 6 * n_in + 37
+    gen = torch.Generator(device="cuda").manual_seed(21)
+    rnd = lambda h, d: torch.randn((1, h, T, d), device="cuda", generator=gen).to(torch.bfloat16)
+    src = [[rnd(r, ds) for _ in range(L * kl)] for _ in range(2)]
+    tgt = [[rnd(1, dt) for _ in range(L)] for _ in range(2)]
+    lmap = [[j * kl + k for k in range(kl)] for j in range(L)]
+    i32 = lambda x: torch.tensor(x, dtype=torch.int32, device="cuda")
+    ws = []
+    for _ in range(3):
+        f = kvx.Fitter(synth.ModelGeom(L * kl, r, ds, 1e4), synth.ModelGeom(L, 1, dt, 1e6), 0.0,
+                       layer_map=lmap if kl > 1 else [m[0] for m in lmap], layers_per_target=kl)
+        f.accumulate(src[0], src[1], i32([T]), i32([0, T]), T, tgt[0], tgt[1])
+        w = [torch.zeros((L, 1, n_in, dt), dtype=torch.bfloat16, device="cuda") for _ in range(2)]
+        assert f.solve(w[0], w[1]) == 0
+        ws.append([x.double().cpu().numpy() for x in w])
+    tol = 2.0 ** -9 + 16 * T * 2.0 ** -24
+    for j in range(L):
+        X = torch.cat([src[1][l][0].permute(1, 0, 2).reshape(T, r * ds) for l in lmap[j]], dim=1).double().cpu().numpy()
+        ref = np.linalg.lstsq(X, tgt[1][j][0, 0].double().cpu().numpy(), rcond=None)[0]
+        for w in ws:
+            assert _rel(w[1][j, 0], ref) <= tol, (j, _rel(w[1][j, 0], ref))
+            assert _rel(w[0][j, 0], ws[0][0][j, 0]) <= 2 * tol, (j, _rel(w[0][j, 0], ws[0][0][j, 0]))
+
+
 def test_fit_two_calls_chunked_and_paged_agree_with_one_call():
     """Sums over calibration calls and accumulation passes add up: one call, two calls, a
     small chunk (several passes) and a paged target cache give the same W (fp32 summation
